@@ -339,13 +339,14 @@ int pwfa_lbm_autotune(pwfa_lbm_t* h, int32_t reps);
  * launches. */
 int pwfa_lbm_set_batching(pwfa_lbm_t* h, int32_t enable);
 
-/* Field-step fusion. For a coupled instance with the rigid driver and a
- * fixed box, the Ampere update of step n (Eq. 5) can run in one kernel with
- * the Faraday update of step n+1: B(t_n+1) is read once for both, and step
- * n+1 starts without its Faraday launch. Results are those of the separate
- * kernels, bit for bit. The kernel-time kind PWFA_KERNEL_AMPERE then covers
- * the fused kernel. Modes: OFF (separate launches), AUTO (the default: fused
- * on grids of 4 Mi nodes or more, where it is faster, and in the batched
+/* Field-step fusion. For a coupled instance with the rigid driver, the
+ * Ampere update of step n (Eq. 5) can run in one kernel with the Faraday
+ * update of step n+1: B(t_n+1) is read once for both, and step n+1 starts
+ * without its Faraday launch (with a moving window, on the steps after which
+ * the box stays). Results are those of the separate kernels, bit for bit.
+ * The kernel-time kind PWFA_KERNEL_AMPERE then covers the fused kernel.
+ * Modes: OFF (separate launches), AUTO (the default: fused on open grids, on
+ * periodic ones from 4 Mi nodes, where it is faster, and in the batched
  * path, whose field launch spans every instance), ON (always);
  * PWFA_ERR_PARAM for another value. In the adjoint sweep the transposed
  * node averages and Faraday update run as one kernel unless the mode is

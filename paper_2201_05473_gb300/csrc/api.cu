@@ -149,8 +149,8 @@ struct pwfa_lbm {
     std::vector<int> pending_kind;            // kind of each recorded pair
     double ms[PWFA_KERNEL_KINDS] = {};
     int64_t launches[PWFA_KERNEL_KINDS] = {};
-    // Ampere fused with the next step's Faraday (rigid driver, no window):
-    // PWFA_FUSION_OFF / _AUTO (grids of kFuseMinNodes and more) / _ON
+    // Ampere fused with the next step's Faraday (rigid driver):
+    // PWFA_FUSION_OFF / _AUTO / _ON (step_fused)
     int field_fusion = PWFA_FUSION_AUTO;
     // batched path (several homogeneous instances, one launch per phase)
     bool batching = true;
@@ -305,18 +305,25 @@ void free_instance(Instance& in) {
     in.arena = nullptr;
 }
 
-// Instances whose Ampere launch can take the next step's Faraday along: the
-// rigid driver (the PIC deposit is cleared by the plain Ampere kernel) and
-// a fixed box (a window move rewrites the B buffer the fused kernel fills).
-bool fusable(const pwfa_lbm_params& p) {
-    return p.couple && p.driver == PWFA_DRIVER_RIGID && !p.moving_window;
-}
+// Instances whose Ampere launch can take the next step's Faraday along: those
+// with the rigid driver (the PIC deposit is cleared by the plain Ampere
+// kernel). A step that the window moves after must not (step_fused).
+bool fusable(const pwfa_lbm_params& p) { return p.couple && p.driver == PWFA_DRIVER_RIGID; }
 
-// The fused kernel marches 16 planes per block, so small grids give it too
-// few blocks: on the GB300 it was slower up to 192x96x96 (1.8 M nodes: 225
-// against 223 us per step; 64x32x32: 27 against 18 us) and faster from
-// 256x128x128 (4.2 M nodes: 485 against 488 us; 512x256x256: 1.2 %).
-constexpr int64_t kFuseMinNodes = (int64_t)4 << 20;
+// Whether the step in hand runs Ampere fused with the next step's Faraday.
+// Automatic mode: always on open grids (step with the regularized FP16 fluid,
+// separate against fused field kernels: 64x32x32 17.6 -> 13.9 us, 96x48x48
+// 28.7 -> 25.2, 128x80x80 79.3 -> 75.2, 256x128x128 308 -> 299); periodic
+// grids have only the tiled kernel, which is slower up to 192x96x96 (225
+// against 223 us per step with the FP32 fluid) and faster from 256x128x128.
+// Before a step that moves the window B must stay at its own time level: the
+// move shifts it, and that step takes its own Faraday launch.
+constexpr int64_t kFuseMinNodesPeriodic = (int64_t)4 << 20;
+bool step_fused(const pwfa_lbm_params& p, const Grid& g, int mode, int64_t steps) {
+    if (!fusable(p) || mode == PWFA_FUSION_OFF) return false;
+    if (mode == PWFA_FUSION_AUTO && g.periodic && g.N < kFuseMinNodesPeriodic) return false;
+    return window_planes_at(p, steps + 2) == window_planes_at(p, steps + 1);
+}
 
 // Zero guard in front of every Yee/current array a step kernel reads: on an
 // open grid the node averages read the -1 neighbours in x, y and z without
@@ -686,9 +693,7 @@ int step_instance(pwfa_lbm* h, Instance& in, const DiagOut* diag) {
         if (rc) return rc;
     }
     in.lookahead = false;
-    const bool fuse = h->field_fusion == PWFA_FUSION_ON ||
-                      (h->field_fusion == PWFA_FUSION_AUTO && in.g.N >= kFuseMinNodes);
-    if (in.p.couple && fuse && fusable(in.p) && in.Ealt[0]) {
+    if (in.Ealt[0] && step_fused(in.p, in.g, h->field_fusion, in.steps)) {
         // Ampere with the next step's Faraday: E into the other E buffer, the
         // next B into the buffer of B(t_n)
         FieldPair out{};

@@ -4,6 +4,7 @@
 // after a state import.
 #include "lbm_kernels.h"
 #include "fields_fused.cuh"
+#include "fields_rows.cuh"
 
 namespace pwfa {
 
@@ -71,6 +72,23 @@ template <bool PER>
 __global__ void __launch_bounds__(kAFX * kAFY, PWFA_AF_MIN_BLOCKS)
     ampere_faraday_kernel(const StepArgs a, const FieldPair out) {
     ampere_faraday_tile<PER>(a, out, blockIdx.x, blockIdx.y, blockIdx.z, a.zc);
+}
+
+// Blocks of four warps, each with its own nodes; eight blocks per SM (64
+// registers): six were slower at every size.
+template <int H>
+__global__ void __launch_bounds__(kARThreads, 8) ampere_faraday_rows_kernel(const StepArgs a, const FieldPair out) {
+    const int n0 = (int)(blockIdx.x * (kARThreads / 32) + (threadIdx.x >> 5)) * kARNodes;
+    if (n0 >= a.g.nx * a.g.ny) return;
+    ampere_faraday_rows<H>(a, out, n0, blockIdx.y * H, a.zc);
+}
+
+template <int H>
+cudaError_t launch_rows(const StepArgs& a, const FieldPair& out, cudaStream_t s) {
+    const int per = kARThreads / 32 * kARNodes;
+    const dim3 grid((unsigned)((a.g.nx * a.g.ny + per - 1) / per), (unsigned)((a.g.nz + H - 1) / H), 1);
+    ampere_faraday_rows_kernel<H><<<grid, kARThreads, 0, s>>>(a, out);
+    return cudaGetLastError();
 }
 
 __global__ void __launch_bounds__(kBX * kBY) zero_walls_kernel(const StepArgs a) {
@@ -172,10 +190,27 @@ void fused_field_tiles(const Grid& g, int* tx, int* ty, int* tz) {
     *tz = (g.nz + kAFZ - 1) / kAFZ;
 }
 
+// Which fused kernel an open grid takes. The z-marching tiles move the least
+// (15 loads a node) and win where DRAM is the limit; below that their
+// blocks of 217 columns x 16 planes are too few or too long, and the rows
+// kernel, with no barrier and any number of planes per warp, is faster
+// (GB300, field update per step, events included, tiles against rows:
+// 512x256x256 396 against 426 us; 384x192x192 177 / 184; 256x128x128 66 / 64;
+// 192x96x96 40 / 32; 128x64x64 19.0 / 14.3; 64x32x32 12.9 / 7.0). More planes per
+// warp reuse more (B of the plane below, J_z of the one above), fewer give
+// more warps: one plane up to 96 Ki nodes (64x32x32: 7.0, 7.8, 8.7 us with 1,
+// 2, 4), two up to 1 Mi (96x48x48: 10.4, 8.7, 10.3), four above
+// (203x97x131: 55, 46, 44).
+constexpr int64_t kRows2Nodes = (int64_t)96 << 10, kRows4Nodes = (int64_t)1 << 20, kTileNodes = (int64_t)8 << 20;
+
 cudaError_t launch_ampere_faraday(const StepArgs& a, const FieldPair& out, cudaStream_t s) {
     if (a.Jb[0]) return cudaErrorInvalidValue;  // the PIC deposit is cleared by the plain Ampere kernel
-    dim3 block(kAFX, kAFY, 1);
-    dim3 grid((a.g.nx + kAFX - 2) / (kAFX - 1), (a.g.ny + kAFY - 2) / (kAFY - 1), (a.g.nz + kAFZ - 1) / kAFZ);
+    if (!a.g.periodic && a.g.N < kTileNodes) {
+        if (a.g.N < kRows2Nodes) return launch_rows<1>(a, out, s);
+        return a.g.N < kRows4Nodes ? launch_rows<2>(a, out, s) : launch_rows<4>(a, out, s);
+    }
+    const dim3 block(kAFX, kAFY, 1);
+    const dim3 grid((a.g.nx + kAFX - 2) / (kAFX - 1), (a.g.ny + kAFY - 2) / (kAFY - 1), (a.g.nz + kAFZ - 1) / kAFZ);
     if (a.g.periodic) ampere_faraday_kernel<true><<<grid, block, 0, s>>>(a, out);
     else ampere_faraday_kernel<false><<<grid, block, 0, s>>>(a, out);
     return cudaGetLastError();

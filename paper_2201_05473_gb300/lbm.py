@@ -392,7 +392,7 @@ class Simulation:
 
     def set_field_fusion(self, mode: int = 1):
         """Ampere fused with the next step's Faraday: FUSION_OFF, FUSION_AUTO
-        (large grids; the default) or FUSION_ON."""
+        (wherever it is faster; the default) or FUSION_ON."""
         _check(self._lib.pwfa_lbm_set_field_fusion(self._h, int(mode)))
 
     def kernel_times(self):
