@@ -369,7 +369,6 @@ def run_ours(args):
             torch.cuda.empty_cache()
             wf = W.production()
             sim = lbm.Simulation(wf, stream=stream)
-            sim.set_launch(*launch_shape)
             barrier()
             with ClockSampler(dev) as fclk:
                 ev0.record(stream)
@@ -486,7 +485,6 @@ def run_ours(args):
             xp, pwt = W.bunch_particles(npart, wp.alpha, wp.sigma_r, wp.sigma_z, wp.z0, wp.dt, wp.nx, wp.ny, wp.dx)
             sp = lbm.Simulation(wp, stream=stream)
             sp.set_particles(xp, pwt)
-            sp.set_launch(*launch_shape)
             sp.step(args.warmup)
             barrier()
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)

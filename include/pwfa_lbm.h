@@ -303,7 +303,8 @@ int pwfa_lbm_profile(pwfa_lbm_t* h, int32_t enable);
 int pwfa_lbm_kernel_times(pwfa_lbm_t* h, double* ms, int64_t* launches);
 
 /* Thread-block shape (bx * by threads, bx along x) of the fused fluid kernel
- * for one instance. bx, by >= 1, bx * by a multiple of 32 and at most 128;
+ * for one instance, in place of the default blocks of 128 consecutive nodes
+ * (which fit any row length; get_launch then reports 64 x 2). bx, by >= 1, bx * by a multiple of 32 and at most 128;
  * PWFA_ERR_PARAM otherwise. */
 int pwfa_lbm_set_launch(pwfa_lbm_t* h, int32_t instance, int32_t bx, int32_t by);
 int pwfa_lbm_get_launch(pwfa_lbm_t* h, int32_t instance, int32_t* bx, int32_t* by);
@@ -319,8 +320,8 @@ int pwfa_lbm_get_launch(pwfa_lbm_t* h, int32_t instance, int32_t* bx, int32_t* b
 int pwfa_lbm_set_fluid_variant(pwfa_lbm_t* h, int32_t instance, int32_t variant);
 int pwfa_lbm_get_fluid_variant(pwfa_lbm_t* h, int32_t instance, int32_t* variant);
 
-/* Autotune the fluid kernel's block shape and variant of every instance: time reps
- * launches (>= 1) of each candidate shape with CUDA events and keep the
+/* Autotune the fluid kernel's blocks and variant of every instance: time reps
+ * launches (>= 1) of each candidate (runs of consecutive nodes, block shapes) with CUDA events and keep the
  * fastest. The kernel is re-run on the current state without advancing it,
  * so the simulation state is unchanged. Synchronises the stream. */
 int pwfa_lbm_autotune(pwfa_lbm_t* h, int32_t reps);

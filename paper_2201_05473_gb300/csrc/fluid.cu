@@ -13,12 +13,22 @@ namespace pwfa {
 
 namespace {
 
+// Blocks of bx x by nodes of a plane (a shape the caller or the autotuner
+// chose).
 template <int ST, int COLL, bool PER>
 __global__ void __launch_bounds__(PWFA_FLUID_MAX_THREADS, FluidOcc<ST, COLL>::blocks) fluid_kernel(const StepArgs a) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= a.g.nx || y >= a.g.ny) return;
     fluid_node<ST, COLL, PER>(a, x, y, blockIdx.z);
+}
+
+// Runs of consecutive nodes (the default).
+template <int ST, int COLL, bool PER>
+__global__ void __launch_bounds__(kLinearThreads, FluidOcc<ST, COLL>::blocks)
+    fluid_linear_kernel(const StepArgs a, const LinearMap m) {
+    int x, y, z;
+    if (m.node(a.g, x, y, z)) fluid_node<ST, COLL, PER>(a, x, y, z);
 }
 
 // The same step with the diagnostics of the entering state fused in: each
@@ -60,13 +70,11 @@ __device__ __forceinline__ float diag8_warp(const float (&v)[8], int lane) {
 }
 
 template <int ST, int COLL, bool PER>
-__global__ void __launch_bounds__(PWFA_FLUID_MAX_THREADS, FluidOcc<ST, COLL>::blocks)
-    fluid_diag_kernel(const StepArgs a, int fields, float* records) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
+__global__ void __launch_bounds__(kLinearThreads, FluidOcc<ST, COLL>::blocks)
+    fluid_diag_kernel(const StepArgs a, const LinearMap m, int fields, float* records) {
+    int x, y, z;
     float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 3.0e38f, 3.0e38f, 0.0f};
-    if (x < a.g.nx && y < a.g.ny) {
+    if (m.node(a.g, x, y, z)) {
         NodeDiag nd;
         fluid_node<ST, COLL, PER, true>(a, x, y, z, &nd);
         if (fields) {
@@ -84,12 +92,10 @@ __global__ void __launch_bounds__(PWFA_FLUID_MAX_THREADS, FluidOcc<ST, COLL>::bl
         v[6] = -nd.beta2;
         v[7] = fin ? 0.0f : 1.0f;
     }
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int lane = tid & 31;
+    const int lane = threadIdx.x & 31;
     const float s = diag8_warp(v, lane);
     if ((lane & 3) == 0) {
-        const int64_t b = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        const int64_t w = b * ((blockDim.x * blockDim.y) >> 5) + (tid >> 5);
+        const int64_t w = (int64_t)blockIdx.x * (kLinearThreads / 32) + (threadIdx.x >> 5);
         records[8 * w + (lane >> 2)] = s;
     }
 }
@@ -236,20 +242,28 @@ template <int ST, int COLL>
 cudaError_t launch_fluid_t(const StepArgs& a, cudaStream_t s, const DiagOut* d) {
     // (a window-moving step pulls one plane up: direct kernel)
     if (a.staged && !d && a.src_shift == 0) return launch_staged_t<ST, COLL>(a, s);
-    const int bx = a.bx, by = a.by;
-    if (bx * by > PWFA_FLUID_MAX_THREADS || bx <= 0 || by <= 0 || (bx * by) % 32) return cudaErrorInvalidConfiguration;
-    dim3 block(bx, by, 1);
-    dim3 grid((a.g.nx + bx - 1) / bx, (a.g.ny + by - 1) / by, a.g.nz);
     if (d) {
-        const int64_t nrec = (int64_t)grid.x * grid.y * grid.z * (bx * by / 32);
+        const int64_t nrec = fluid_diag_records(a.g);
         if (nrec > d->capacity) return cudaErrorInvalidValue;
         const int fields = d->nenergy > 0 ? 0 : 1;
-        if (a.g.periodic) fluid_diag_kernel<ST, COLL, true><<<grid, block, 0, s>>>(a, fields, d->records);
-        else fluid_diag_kernel<ST, COLL, false><<<grid, block, 0, s>>>(a, fields, d->records);
+        const LinearMap m(a.g);
+        if (a.g.periodic)
+            fluid_diag_kernel<ST, COLL, true><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m, fields, d->records);
+        else fluid_diag_kernel<ST, COLL, false><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m, fields, d->records);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         return launch_diag_finish_step(*d, nrec, s);
     }
+    if (a.linear) {
+        const LinearMap m(a.g);
+        if (a.g.periodic) fluid_linear_kernel<ST, COLL, true><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m);
+        else fluid_linear_kernel<ST, COLL, false><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m);
+        return cudaGetLastError();
+    }
+    const int bx = a.bx, by = a.by;
+    if (bx * by > PWFA_FLUID_MAX_THREADS || bx <= 0 || by <= 0 || (bx * by) % 32) return cudaErrorInvalidConfiguration;
+    dim3 block(bx, by, 1);
+    dim3 grid((a.g.nx + bx - 1) / bx, (a.g.ny + by - 1) / by, a.g.nz);
     if (a.g.periodic) fluid_kernel<ST, COLL, true><<<grid, block, 0, s>>>(a);
     else fluid_kernel<ST, COLL, false><<<grid, block, 0, s>>>(a);
     return cudaGetLastError();
@@ -266,6 +280,8 @@ cudaError_t launch_fluid_s(const StepArgs& a, int collision, cudaStream_t s, con
 }
 
 }  // namespace
+
+int64_t fluid_diag_records(const Grid& g) { return (int64_t)linear_blocks(g) * (kLinearThreads / 32); }
 
 cudaError_t launch_fluid(const StepArgs& a, int storage, int collision, cudaStream_t s, const DiagOut* d) {
     switch (storage) {

@@ -10,22 +10,18 @@ namespace pwfa {
 namespace {
 
 template <int ST, int COLL, bool PER>
-__global__ void __launch_bounds__(PWFA_FLUID_MAX_THREADS, FluidOcc<ST, COLL>::blocks) fluid_mom_kernel(const StepArgs a) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= a.g.nx || y >= a.g.ny) return;
-    fluid_node<ST, COLL, PER, false, true>(a, x, y, blockIdx.z);
+__global__ void __launch_bounds__(kLinearThreads, FluidOcc<ST, COLL>::blocks)
+    fluid_mom_kernel(const StepArgs a, const LinearMap m) {
+    int x, y, z;
+    if (m.node(a.g, x, y, z)) fluid_node<ST, COLL, PER, false, true>(a, x, y, z);
 }
 
 template <int ST, int COLL>
 cudaError_t launch_t(const StepArgs& a, cudaStream_t s) {
-    const int bx = a.bx, by = a.by;
-    if (bx * by > PWFA_FLUID_MAX_THREADS || bx <= 0 || by <= 0 || (bx * by) % 32 || !a.mom)
-        return cudaErrorInvalidConfiguration;
-    dim3 block(bx, by, 1);
-    dim3 grid((a.g.nx + bx - 1) / bx, (a.g.ny + by - 1) / by, a.g.nz);
-    if (a.g.periodic) fluid_mom_kernel<ST, COLL, true><<<grid, block, 0, s>>>(a);
-    else fluid_mom_kernel<ST, COLL, false><<<grid, block, 0, s>>>(a);
+    if (!a.mom) return cudaErrorInvalidConfiguration;
+    const LinearMap m(a.g);
+    if (a.g.periodic) fluid_mom_kernel<ST, COLL, true><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m);
+    else fluid_mom_kernel<ST, COLL, false><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m);
     return cudaGetLastError();
 }
 

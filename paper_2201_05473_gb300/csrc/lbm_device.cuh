@@ -179,6 +179,20 @@ __host__ __device__ __forceinline__ int64_t pop_elem(int l, uint32_t off, int64_
     return ST == 0 ? (int64_t)l * LS + off : (int64_t)(l >> 1) * 2 * LS + 2 * (int64_t)off + (l & 1);
 }
 
+// Division of 0 <= n < 2^31 by a number known on the host, as a
+// multiplication and a shift.
+struct FastDiv {
+    uint32_t d, m, s;
+    FastDiv() = default;
+    explicit FastDiv(uint32_t d_) : d(d_), m(0), s(0) {
+        while (((uint64_t)1 << s) < d) ++s;
+        m = (uint32_t)((((uint64_t)1 << 32) * (((uint64_t)1 << s) - d)) / d + 1);
+    }
+#ifdef __CUDACC__
+    __device__ __forceinline__ uint32_t div(uint32_t n) const { return (__umulhi(n, m) + n) >> s; }
+#endif
+};
+
 // One instance's device state as the step kernels see it.
 struct StepArgs {
     Grid g;
@@ -208,6 +222,7 @@ struct StepArgs {
                           // that moves the window (the streaming source is
                           // read one plane up), else 0
     int bx, by;           // fluid kernel block shape (autotuned per instance)
+    int linear;           // 1: blocks of 128 consecutive nodes instead of bx x by (LinearMap)
     int staged;           // 1: software-pipelined fluid kernel (FP32 storage), 128-thread tiles
     unsigned* dbg;        // debug builds: the instance's index-error word (see PWFA_CHECK)
     float* mom;           // adjoint recompute (launch_fluid_mom): each node's lattice

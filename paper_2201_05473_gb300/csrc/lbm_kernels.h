@@ -71,6 +71,9 @@ struct DiagOut {
 cudaError_t launch_fluid(const StepArgs& a, int storage, int collision, cudaStream_t s,
                          const DiagOut* d = nullptr);
 
+// FP32 records of 8 values that launch_fluid writes with d != NULL.
+int64_t fluid_diag_records(const Grid& g);
+
 // The same fluid step that also stores each node's lattice sums A_l into
 // a.mom ([4][N] FP32): the adjoint's recomputed forward steps keep them for
 // the reverse step, which needs nothing else of the populations.
