@@ -16,6 +16,7 @@
 // with c = dt/dx. All adjoint state is FP32; parameter gradients are FP64.
 #include "lbm_adjoint.h"
 #include "lbm_node.cuh"
+#include "launch.cuh"
 
 namespace pwfa {
 
@@ -181,6 +182,7 @@ constexpr int kR1Planes = 2;
 
 template <bool PER>
 __global__ void __launch_bounds__(kBX * kBY) adj_ampere_kernel(const AdjArgs a) {
+    chain_begin();
     const Grid& g = a.f.g;
     const int i = blockIdx.x * kBX + threadIdx.x;
     const int j = blockIdx.y * kBY + threadIdx.y;
@@ -288,6 +290,7 @@ __device__ __forceinline__ void shell_node(const Grid& g, uint32_t idx, int& x, 
 template <int ST, int COLL, bool PER, bool SHELL>
 __global__ void __launch_bounds__(kAdjThreads, PWFA_ADJ_MIN_BLOCKS) adj_fluid_kernel(const AdjArgs a,
                                                                                     uint32_t nshell) {
+    chain_begin();
     using T = typename Codec<ST>::T;
     __shared__ float sA[kL][32];     // lattice sums A_l
     __shared__ float sG[kL][32];     // sum_i w_i S_bar_l,i
@@ -739,6 +742,7 @@ __device__ __forceinline__ void adj_fe_load(const AdjArgs& a, int o, int pi, int
 
 template <bool PER>
 __global__ void __launch_bounds__(kRX * kRY, PWFA_ADJ_FE_MIN_BLOCKS) adj_faces_edges_kernel(const AdjArgs a) {
+    chain_begin();
     const Grid& g = a.f.g;
     const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
     __shared__ float sBx[2][kRY][kRX], sBz[2][kRY][kRX];
@@ -895,15 +899,12 @@ cudaError_t launch_adj_fluid_t(const AdjArgs& a, cudaStream_t s) {
     const Grid& g = a.f.g;
     const dim3 rows((unsigned)(g.nx + 31) / 32, (unsigned)g.ny, (unsigned)g.nz);
     if (g.periodic) {
-        adj_fluid_kernel<ST, COLL, true, false><<<rows, kAdjThreads, 0, s>>>(a, 0u);
-    } else {
-        const uint32_t nb = shell_count(g);
-        adj_fluid_kernel<ST, COLL, false, true><<<(nb + 31) / 32, kAdjThreads, 0, s>>>(a, nb);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        adj_fluid_kernel<ST, COLL, false, false><<<rows, kAdjThreads, 0, s>>>(a, 0u);
+        return launch_chained(adj_fluid_kernel<ST, COLL, true, false>, rows, kAdjThreads, s, a, 0u);
     }
-    return cudaGetLastError();
+    const uint32_t nb = shell_count(g);
+    cudaError_t e = launch_chained(adj_fluid_kernel<ST, COLL, false, true>, (nb + 31) / 32, kAdjThreads, s, a, nb);
+    if (e != cudaSuccess) return e;
+    return launch_chained(adj_fluid_kernel<ST, COLL, false, false>, rows, kAdjThreads, s, a, 0u);
 }
 
 template <int ST>
@@ -936,16 +937,13 @@ cudaError_t launch_adjoint_ampere(const AdjArgs& a0, cudaStream_t s) {
     const dim3 block(kBX, kBY, 1);
     const dim3 grid((g.nx + kBX - 1) / kBX, (g.ny + kBY - 1) / kBY, (g.nz + kR1Planes - 1) / kR1Planes);
     if (a.f.couple) {
-        if (g.periodic) adj_ampere_kernel<true><<<grid, block, 0, s>>>(a);
-        else adj_ampere_kernel<false><<<grid, block, 0, s>>>(a);
-    } else {
-        // no Maxwell update: B, E pass through; J is not used
-        cudaError_t e = cudaMemsetAsync(a.Jbar[0], 0, sizeof(float) * g.N, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(a.Jbar[1], 0, sizeof(float) * g.N, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(a.Jbar[2], 0, sizeof(float) * g.N, s);
-        if (e != cudaSuccess) return e;
+        return launch_chained(g.periodic ? adj_ampere_kernel<true> : adj_ampere_kernel<false>, grid, block, s, a);
     }
-    return cudaGetLastError();
+    // no Maxwell update: B, E pass through; J is not used
+    cudaError_t e = cudaMemsetAsync(a.Jbar[0], 0, sizeof(float) * g.N, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.Jbar[1], 0, sizeof(float) * g.N, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.Jbar[2], 0, sizeof(float) * g.N, s);
+    return e;
 }
 
 cudaError_t launch_adjoint_fluid(const AdjArgs& a0, int storage, int collision, cudaStream_t s) {
@@ -967,9 +965,7 @@ cudaError_t launch_adjoint_fields(const AdjArgs& a0, bool fused, cudaStream_t s)
         const dim3 tiles((unsigned)(g.nx + kRX - 2) / (kRX - 1), (unsigned)(g.ny + kRY - 2) / (kRY - 1),
                          (unsigned)(g.nz + kRZ - 1) / kRZ);
         const dim3 block(kRX, kRY, 1);
-        if (per) adj_faces_edges_kernel<true><<<tiles, block, 0, s>>>(a);
-        else adj_faces_edges_kernel<false><<<tiles, block, 0, s>>>(a);
-        return cudaGetLastError();
+        return launch_chained(per ? adj_faces_edges_kernel<true> : adj_faces_edges_kernel<false>, tiles, block, s, a);
     }
     const dim3 grid = grid_of(g, kBX, kBY), block(kBX, kBY, 1);
     if (per) adj_faces_kernel<true><<<grid, block, 0, s>>>(a);

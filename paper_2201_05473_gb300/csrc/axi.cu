@@ -3,6 +3,7 @@
 // with the driver, and the node moments for exports. One thread per node,
 // warps along r (coalesced rows).
 #include "axi.h"
+#include "launch.cuh"
 
 namespace pwfa {
 namespace axi {
@@ -96,6 +97,7 @@ constexpr int kOut = 30;  // output nodes per warp
 #define PWFA_AXI_MIN_BLOCKS 7
 #endif
 __global__ void __launch_bounds__(kBR * kBZ, PWFA_AXI_MIN_BLOCKS) fluid_kernel(const Args a) {
+    chain_begin();
     const int lane = (int)threadIdx.x;
     const int j = (int)blockIdx.x * kOut + lane - 1;
     const int k = (int)(blockIdx.y * kBZ + threadIdx.y);
@@ -218,6 +220,7 @@ __global__ void __launch_bounds__(kBR * kBZ, PWFA_AXI_MIN_BLOCKS) fluid_kernel(c
 
 // Ampere: dE_r/dt = -dB_theta/dz - J_r, dE_z/dt = (1/r) d(r B_theta)/dr - J_z - J_b
 __global__ void __launch_bounds__(kBR * kBZ) ampere_kernel(const Args a) {
+    chain_begin();
     const int j = blockIdx.x * kBR + threadIdx.x;
     const int k = blockIdx.y * kBZ + threadIdx.y;
     if (j >= a.nr || k >= a.nz) return;
@@ -269,12 +272,10 @@ cudaError_t launch_moments(const Args& a, cudaStream_t s) {
 }
 cudaError_t launch_fluid(const Args& a, cudaStream_t s) {
     const dim3 grid((unsigned)((a.nr + kOut - 1) / kOut), (unsigned)((a.nz + kBZ - 1) / kBZ), 1);
-    fluid_kernel<<<grid, dim3(kBR, kBZ), 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fluid_kernel, grid, dim3(kBR, kBZ), s, a);
 }
 cudaError_t launch_ampere(const Args& a, cudaStream_t s) {
-    ampere_kernel<<<grid_of(a), dim3(kBR, kBZ), 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(ampere_kernel, grid_of(a), dim3(kBR, kBZ), s, a);
 }
 cudaError_t launch_init(const Args& a, float* f, cudaStream_t s) {
     const int64_t n = (int64_t)kL * kQ * a.Np;

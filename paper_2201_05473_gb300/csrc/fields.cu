@@ -5,6 +5,7 @@
 #include "lbm_kernels.h"
 #include "fields_fused.cuh"
 #include "fields_rows.cuh"
+#include "launch.cuh"
 
 namespace pwfa {
 
@@ -24,6 +25,7 @@ constexpr int kBY = PWFA_FIELD_BY;
 
 template <bool PER>
 __global__ void __launch_bounds__(kBX * kBY) faraday_kernel(const StepArgs a) {
+    chain_begin();
     const int i = blockIdx.x * kBX + threadIdx.x;
     const int j = blockIdx.y * kBY + threadIdx.y;
     if (i >= a.g.nx || j >= a.g.ny) return;
@@ -57,6 +59,7 @@ __global__ void __launch_bounds__(kBX * kBY) faraday_energy_kernel(const StepArg
 
 template <bool PER>
 __global__ void __launch_bounds__(kBX * kBY) ampere_kernel(const StepArgs a) {
+    chain_begin();
     const int i = blockIdx.x * kBX + threadIdx.x;
     const int j = blockIdx.y * kBY + threadIdx.y;
     if (a.jbox_next && i == 0 && j == 0 && blockIdx.z == 0) {
@@ -71,6 +74,7 @@ __global__ void __launch_bounds__(kBX * kBY) ampere_kernel(const StepArgs a) {
 template <bool PER>
 __global__ void __launch_bounds__(kAFX * kAFY, PWFA_AF_MIN_BLOCKS)
     ampere_faraday_kernel(const StepArgs a, const FieldPair out) {
+    chain_begin();
     ampere_faraday_tile<PER>(a, out, blockIdx.x, blockIdx.y, blockIdx.z, a.zc);
 }
 
@@ -78,6 +82,7 @@ __global__ void __launch_bounds__(kAFX * kAFY, PWFA_AF_MIN_BLOCKS)
 // registers): six were slower at every size.
 template <int H>
 __global__ void __launch_bounds__(kARThreads, 8) ampere_faraday_rows_kernel(const StepArgs a, const FieldPair out) {
+    chain_begin();
     const int n0 = (int)(blockIdx.x * (kARThreads / 32) + (threadIdx.x >> 5)) * kARNodes;
     if (n0 >= a.g.nx * a.g.ny) return;
     ampere_faraday_rows<H>(a, out, n0, blockIdx.y * H, a.zc);
@@ -87,8 +92,7 @@ template <int H>
 cudaError_t launch_rows(const StepArgs& a, const FieldPair& out, cudaStream_t s) {
     const int per = kARThreads / 32 * kARNodes;
     const dim3 grid((unsigned)((a.g.nx * a.g.ny + per - 1) / per), (unsigned)((a.g.nz + H - 1) / H), 1);
-    ampere_faraday_rows_kernel<H><<<grid, kARThreads, 0, s>>>(a, out);
-    return cudaGetLastError();
+    return launch_chained(ampere_faraday_rows_kernel<H>, grid, kARThreads, s, a, out);
 }
 
 __global__ void __launch_bounds__(kBX * kBY) zero_walls_kernel(const StepArgs a) {
@@ -179,9 +183,9 @@ cudaError_t launch_faraday(const StepArgs& a, cudaStream_t s, float* energy) {
     if (energy) {
         if (a.g.periodic) faraday_energy_kernel<true><<<grid, block, 0, s>>>(a, energy);
         else faraday_energy_kernel<false><<<grid, block, 0, s>>>(a, energy);
-    } else if (a.g.periodic) faraday_kernel<true><<<grid, block, 0, s>>>(a);
-    else faraday_kernel<false><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+        return cudaGetLastError();
+    }
+    return launch_chained(a.g.periodic ? faraday_kernel<true> : faraday_kernel<false>, grid, block, s, a);
 }
 
 void fused_field_tiles(const Grid& g, int* tx, int* ty, int* tz) {
@@ -211,17 +215,14 @@ cudaError_t launch_ampere_faraday(const StepArgs& a, const FieldPair& out, cudaS
     }
     const dim3 block(kAFX, kAFY, 1);
     const dim3 grid((a.g.nx + kAFX - 2) / (kAFX - 1), (a.g.ny + kAFY - 2) / (kAFY - 1), (a.g.nz + kAFZ - 1) / kAFZ);
-    if (a.g.periodic) ampere_faraday_kernel<true><<<grid, block, 0, s>>>(a, out);
-    else ampere_faraday_kernel<false><<<grid, block, 0, s>>>(a, out);
-    return cudaGetLastError();
+    return launch_chained(a.g.periodic ? ampere_faraday_kernel<true> : ampere_faraday_kernel<false>, grid, block, s, a,
+                          out);
 }
 
 cudaError_t launch_ampere(const StepArgs& a, cudaStream_t s) {
     dim3 block(kBX, kBY, 1);
     dim3 grid((a.g.nx + kBX - 1) / kBX, (a.g.ny + kBY - 1) / kBY, a.g.nz);
-    if (a.g.periodic) ampere_kernel<true><<<grid, block, 0, s>>>(a);
-    else ampere_kernel<false><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(a.g.periodic ? ampere_kernel<true> : ampere_kernel<false>, grid, block, s, a);
 }
 
 }  // namespace pwfa

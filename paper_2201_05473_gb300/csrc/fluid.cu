@@ -8,6 +8,7 @@
 
 #include "lbm_kernels.h"
 #include "fluid_node.cuh"
+#include "launch.cuh"
 
 namespace pwfa {
 
@@ -27,6 +28,7 @@ __global__ void __launch_bounds__(PWFA_FLUID_MAX_THREADS, FluidOcc<ST, COLL>::bl
 template <int ST, int COLL, bool PER>
 __global__ void __launch_bounds__(kLinearThreads, FluidOcc<ST, COLL>::blocks)
     fluid_linear_kernel(const StepArgs a, const LinearMap m) {
+    chain_begin();
     int x, y, z;
     if (m.node(a.g, x, y, z)) fluid_node<ST, COLL, PER>(a, x, y, z);
 }
@@ -72,6 +74,7 @@ __device__ __forceinline__ float diag8_warp(const float (&v)[8], int lane) {
 template <int ST, int COLL, bool PER>
 __global__ void __launch_bounds__(kLinearThreads, FluidOcc<ST, COLL>::blocks)
     fluid_diag_kernel(const StepArgs a, const LinearMap m, int fields, float* records) {
+    chain_begin();
     int x, y, z;
     float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 3.0e38f, 3.0e38f, 0.0f};
     if (m.node(a.g, x, y, z)) {
@@ -247,19 +250,16 @@ cudaError_t launch_fluid_t(const StepArgs& a, cudaStream_t s, const DiagOut* d) 
         if (nrec > d->capacity) return cudaErrorInvalidValue;
         const int fields = d->nenergy > 0 ? 0 : 1;
         const LinearMap m(a.g);
-        if (a.g.periodic)
-            fluid_diag_kernel<ST, COLL, true><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m, fields, d->records);
-        else fluid_diag_kernel<ST, COLL, false><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m, fields, d->records);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = launch_chained(
+            a.g.periodic ? fluid_diag_kernel<ST, COLL, true> : fluid_diag_kernel<ST, COLL, false>, linear_blocks(a.g),
+            kLinearThreads, s, a, m, fields, d->records);
         if (e != cudaSuccess) return e;
         return launch_diag_finish_step(*d, nrec, s);
     }
-    if (a.linear) {
-        const LinearMap m(a.g);
-        if (a.g.periodic) fluid_linear_kernel<ST, COLL, true><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m);
-        else fluid_linear_kernel<ST, COLL, false><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m);
-        return cudaGetLastError();
-    }
+    if (a.linear)
+        return launch_chained(
+            a.g.periodic ? fluid_linear_kernel<ST, COLL, true> : fluid_linear_kernel<ST, COLL, false>,
+            linear_blocks(a.g), kLinearThreads, s, a, LinearMap(a.g));
     const int bx = a.bx, by = a.by;
     if (bx * by > PWFA_FLUID_MAX_THREADS || bx <= 0 || by <= 0 || (bx * by) % 32) return cudaErrorInvalidConfiguration;
     dim3 block(bx, by, 1);

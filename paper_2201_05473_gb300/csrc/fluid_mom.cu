@@ -4,6 +4,7 @@
 // build is unchanged).
 #include "lbm_kernels.h"
 #include "fluid_node.cuh"
+#include "launch.cuh"
 
 namespace pwfa {
 
@@ -12,6 +13,7 @@ namespace {
 template <int ST, int COLL, bool PER>
 __global__ void __launch_bounds__(kLinearThreads, FluidOcc<ST, COLL>::blocks)
     fluid_mom_kernel(const StepArgs a, const LinearMap m) {
+    chain_begin();
     int x, y, z;
     if (m.node(a.g, x, y, z)) fluid_node<ST, COLL, PER, false, true>(a, x, y, z);
 }
@@ -19,10 +21,8 @@ __global__ void __launch_bounds__(kLinearThreads, FluidOcc<ST, COLL>::blocks)
 template <int ST, int COLL>
 cudaError_t launch_t(const StepArgs& a, cudaStream_t s) {
     if (!a.mom) return cudaErrorInvalidConfiguration;
-    const LinearMap m(a.g);
-    if (a.g.periodic) fluid_mom_kernel<ST, COLL, true><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m);
-    else fluid_mom_kernel<ST, COLL, false><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m);
-    return cudaGetLastError();
+    return launch_chained(a.g.periodic ? fluid_mom_kernel<ST, COLL, true> : fluid_mom_kernel<ST, COLL, false>,
+                          linear_blocks(a.g), kLinearThreads, s, a, LinearMap(a.g));
 }
 
 template <int ST>

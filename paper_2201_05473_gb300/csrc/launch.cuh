@@ -1,0 +1,37 @@
+// Launches of a chain of kernels on one stream, each overlapping its start
+// with the tail of the one before (programmatic dependent launch).
+//
+// A chained kernel calls chain_begin() before it touches global memory. The
+// hardware may bring its blocks up once every block of the kernel before has
+// started, and holds them in chain_begin until that kernel has completed and
+// its writes are visible: the same order as a plain launch, without the
+// launch latency and the ramp between the two. Behind a kernel that is not
+// chained, a copy or an event the launch is ordered as usual.
+#pragma once
+
+#include <utility>
+
+#include <cuda_runtime.h>
+
+namespace pwfa {
+
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A&&... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
+}  // namespace pwfa
