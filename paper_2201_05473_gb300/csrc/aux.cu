@@ -6,6 +6,7 @@ namespace pwfa {
 
 namespace {
 
+// blocks of the field export
 constexpr int kBX = 32;
 constexpr int kBY = 4;
 
@@ -63,13 +64,11 @@ __global__ void init_kernel(Grid g, typename Codec<ST>::T* f, float n0, const do
 
 // f^n at every node (boundary nodes: f^eq of the clamped interior node).
 template <int ST, bool PER>
-__global__ void __launch_bounds__(kBX * kBY) export_f_kernel(const StepArgs a, float* out) {
+__global__ void __launch_bounds__(kLinearThreads) export_f_kernel(const StepArgs a, const LinearMap m, float* out) {
     using T = typename Codec<ST>::T;
     const Grid& g = a.g;
-    const int x = blockIdx.x * kBX + threadIdx.x;
-    const int y = blockIdx.y * kBY + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= g.nx || y >= g.ny) return;
+    int x, y, z;
+    if (!m.node(g, x, y, z)) return;
     const int64_t node = ((int64_t)z * g.ny + y) * g.nx + x;
     float f[kL][kQ];
     bool bnd;
@@ -88,22 +87,45 @@ __global__ void __launch_bounds__(kBX * kBY) export_f_kernel(const StepArgs a, f
         for (int q = 0; q < kQ; ++q) out[(int64_t)(l * kQ + q) * g.N + node] = f[l][q];
 }
 
-// Inverse of the pull: S_i(y) = f^n_i(y + xi_i).
-template <int ST>
-__global__ void import_f_kernel(Grid g, const float* in, typename Codec<ST>::T* f, float n0) {
-    const int64_t node = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (node >= g.N) return;
+// Inverse of the pull: S_i(y) = f^n_i(y + xi_i). A block takes 128 consecutive
+// nodes and one pair of lattices (blockIdx.y), and a thread issues its 38
+// loads before any store: DRAM-bound (608 B/node FP32). One population after
+// another had left a single round of four loads in flight per thread:
+// 256x128x128 FP32 set_state 773 -> 464 us.
+template <int ST, bool PER>
+__global__ void __launch_bounds__(kLinearThreads) import_f_kernel(Grid g, const LinearMap m,
+                                                                  const float* __restrict__ in,
+                                                                  typename Codec<ST>::T* f, float n0) {
     int x, y, z;
-    node_xyz(g, node, x, y, z);
-#pragma unroll 1
+    if (!m.node(g, x, y, z)) return;
+    const int64_t node = ((int64_t)z * g.ny + y) * g.nx + x;
+    // offsets to the neighbours, wrapped or clamped into the grid
+    const int64_t sx = g.nx, sxy = sx * g.ny;
+    const int64_t ox[3] = {x > 0 ? -1 : (PER ? g.nx - 1 : 0), 0, x < g.nx - 1 ? 1 : (PER ? 1 - g.nx : 0)};
+    const int64_t oy[3] = {y > 0 ? -sx : (PER ? (g.ny - 1) * sx : 0), 0, y < g.ny - 1 ? sx : (PER ? (1 - g.ny) * sx : 0)};
+    const int64_t oz[3] = {z > 0 ? -sxy : (PER ? (g.nz - 1) * sxy : 0), 0,
+                           z < g.nz - 1 ? sxy : (PER ? (1 - g.nz) * sxy : 0)};
+    const int l0 = 2 * (int)blockIdx.y;
+    const float* p0 = in + (int64_t)l0 * kQ * g.N + node;
+    const float* p1 = p0 + (int64_t)kQ * g.N;
+    float v0[kQ], v1[kQ];
+#pragma unroll
     for (int q = 0; q < kQ; ++q) {
-        int sx = x + xi_x(q), sy = y + xi_y(q), sz = z + xi_z(q);
-        if (g.periodic) { sx = wrapi(sx, g.nx); sy = wrapi(sy, g.ny); sz = wrapi(sz, g.nz); }
-        else { sx = min(max(sx, 0), g.nx - 1); sy = min(max(sy, 0), g.ny - 1); sz = min(max(sz, 0), g.nz - 1); }
-        const int64_t src = ((int64_t)sz * g.ny + sy) * g.nx + sx;
-        for (int l = 0; l < kL; ++l)
-            Codec<ST>::store(f + pop_elem<ST>(l, pop_off(q, (uint32_t)node), lattice_stride(g)),
-                             in[(int64_t)(l * kQ + q) * g.N + src], l, q, n0);
+        const int64_t o = q * g.N + ox[xi_x(q) + 1] + oy[xi_y(q) + 1] + oz[xi_z(q) + 1];
+        v0[q] = __ldg(p0 + o);
+        v1[q] = __ldg(p1 + o);
+    }
+    const int64_t LS = lattice_stride(g);
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) {
+        const uint32_t off = pop_off(q, (uint32_t)node);
+        auto* d = f + pop_elem<ST>(l0, off, LS);
+        if constexpr (ST == 0) {
+            Codec<ST>::store(d, v0[q], l0, q, n0);
+            Codec<ST>::store(d + LS, v1[q], l0 + 1, q, n0);
+        } else {
+            Codec<ST>::store2(d, v0[q], v1[q], l0, q, n0);
+        }
     }
 }
 
@@ -276,8 +298,6 @@ __global__ void __launch_bounds__(kDiagThreads) diag_chunk_kernel(const float* r
     diag_block_reduce(d, scratch + 8 * (int64_t)blockIdx.x);
 }
 
-dim3 node_grid(const Grid& g) { return dim3((g.nx + kBX - 1) / kBX, (g.ny + kBY - 1) / kBY, g.nz); }
-
 // Witness slab: the x range [rows[2 j], rows[2 j + 1]) of each row j in plane
 // k. One block sums E_z over it in FP64 (the slab holds at most a few
 // thousand edges).
@@ -348,40 +368,56 @@ cudaError_t launch_init(const Grid& g, void* f, int storage, float n0, const dou
     return cudaGetLastError();
 }
 
+template <int ST>
+static cudaError_t export_f(const StepArgs& a, float* out, cudaStream_t s) {
+    const LinearMap m(a.g);
+    if (a.g.periodic) export_f_kernel<ST, true><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m, out);
+    else export_f_kernel<ST, false><<<linear_blocks(a.g), kLinearThreads, 0, s>>>(a, m, out);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_export_f(const StepArgs& a, int storage, float* out, cudaStream_t s) {
-    const dim3 grid = node_grid(a.g), block(kBX, kBY, 1);
-    const bool per = a.g.periodic;
     switch (storage) {
-        case 0: if (per) export_f_kernel<0, true><<<grid, block, 0, s>>>(a, out); else export_f_kernel<0, false><<<grid, block, 0, s>>>(a, out); break;
-        case 1: if (per) export_f_kernel<1, true><<<grid, block, 0, s>>>(a, out); else export_f_kernel<1, false><<<grid, block, 0, s>>>(a, out); break;
-        case 2: if (per) export_f_kernel<2, true><<<grid, block, 0, s>>>(a, out); else export_f_kernel<2, false><<<grid, block, 0, s>>>(a, out); break;
-        default: return cudaErrorInvalidValue;
+        case 0: return export_f<0>(a, out, s);
+        case 1: return export_f<1>(a, out, s);
+        case 2: return export_f<2>(a, out, s);
     }
+    return cudaErrorInvalidValue;
+}
+
+template <int ST>
+static cudaError_t import_f(const Grid& g, const float* in, void* f, float n0, cudaStream_t s) {
+    using T = typename Codec<ST>::T;
+    const dim3 grid(linear_blocks(g), kL / 2, 1);
+    if (g.periodic) import_f_kernel<ST, true><<<grid, kLinearThreads, 0, s>>>(g, LinearMap(g), in, static_cast<T*>(f), n0);
+    else import_f_kernel<ST, false><<<grid, kLinearThreads, 0, s>>>(g, LinearMap(g), in, static_cast<T*>(f), n0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_import_f(const Grid& g, const float* in, void* f, int storage, float n0, cudaStream_t s) {
-    const int threads = 256;
-    const unsigned blocks = (unsigned)((g.N + threads - 1) / threads);
     switch (storage) {
-        case 0: import_f_kernel<0><<<blocks, threads, 0, s>>>(g, in, (float*)f, n0); break;
-        case 1: import_f_kernel<1><<<blocks, threads, 0, s>>>(g, in, (__nv_bfloat16*)f, n0); break;
-        case 2: import_f_kernel<2><<<blocks, threads, 0, s>>>(g, in, (__half*)f, n0); break;
-        default: return cudaErrorInvalidValue;
+        case 0: return import_f<0>(g, in, f, n0, s);
+        case 1: return import_f<1>(g, in, f, n0, s);
+        case 2: return import_f<2>(g, in, f, n0, s);
     }
+    return cudaErrorInvalidValue;
+}
+
+template <int ST>
+static cudaError_t export_fields(const StepArgs& a, unsigned mask, float* out, cudaStream_t s) {
+    const dim3 grid((a.g.nx + kBX - 1) / kBX, (a.g.ny + kBY - 1) / kBY, a.g.nz), block(kBX, kBY, 1);
+    if (a.g.periodic) export_fields_kernel<ST, true><<<grid, block, 0, s>>>(a, mask, out);
+    else export_fields_kernel<ST, false><<<grid, block, 0, s>>>(a, mask, out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_export_fields(const StepArgs& a, int storage, unsigned mask, float* out, cudaStream_t s) {
-    const dim3 grid = node_grid(a.g), block(kBX, kBY, 1);
-    const bool per = a.g.periodic;
     switch (storage) {
-        case 0: if (per) export_fields_kernel<0, true><<<grid, block, 0, s>>>(a, mask, out); else export_fields_kernel<0, false><<<grid, block, 0, s>>>(a, mask, out); break;
-        case 1: if (per) export_fields_kernel<1, true><<<grid, block, 0, s>>>(a, mask, out); else export_fields_kernel<1, false><<<grid, block, 0, s>>>(a, mask, out); break;
-        case 2: if (per) export_fields_kernel<2, true><<<grid, block, 0, s>>>(a, mask, out); else export_fields_kernel<2, false><<<grid, block, 0, s>>>(a, mask, out); break;
-        default: return cudaErrorInvalidValue;
+        case 0: return export_fields<0>(a, mask, out, s);
+        case 1: return export_fields<1>(a, mask, out, s);
+        case 2: return export_fields<2>(a, mask, out, s);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_linecut(const StepArgs& a, int storage, double r, float* out, cudaStream_t s) {

@@ -17,33 +17,7 @@
 
 namespace pwfa {
 
-// Nodes as runs of consecutive indices: block b of a fluid kernel takes nodes
-// [128 b, 128 b + 128) of the [z][y][x] order, four whole chunks of the
-// population layout. No lane idles and no store is misaligned whatever the
-// row length (a 64 x 2 block on rows of 131 nodes works with 131 of 192
-// lanes), and even on rows that blocks fit the own-node accesses of a block
-// are one contiguous piece. Fluid kernel on GB300, 64 x 2 blocks against
-// runs: 203x97x131 BGK FP32 303 -> 255 us, regularized FP16 178 -> 149;
-// 160x100x96 165 -> 153; 256x128x128 BGK 414 -> 409, regularized 399 both;
-// 512x256x256 BGK 3265 -> 3226, regularized 3169 / 3174, FP16 1842 -> 1817;
-// 64x32x32 11.8 -> 10.3.
-constexpr int kLinearThreads = 128;
 static_assert(kLinearThreads <= PWFA_FLUID_MAX_THREADS, "launch bounds");
-struct LinearMap {
-    FastDiv nxy, nx;
-    explicit LinearMap(const Grid& g) : nxy((uint32_t)g.nx * (uint32_t)g.ny), nx((uint32_t)g.nx) {}
-    // false: past the last node
-    __device__ __forceinline__ bool node(const Grid& g, int& x, int& y, int& z) const {
-        const uint32_t n = blockIdx.x * kLinearThreads + threadIdx.x;
-        if (n >= (uint32_t)g.N) return false;
-        const uint32_t k = nxy.div(n), r = n - k * nxy.d, j = nx.div(r);
-        x = (int)(r - j * nx.d);
-        y = (int)j;
-        z = (int)k;
-        return true;
-    }
-};
-inline unsigned linear_blocks(const Grid& g) { return (unsigned)((g.N + kLinearThreads - 1) / kLinearThreads); }
 
 // Node quantities handed to the fused diagnostics (state entering the step).
 struct NodeDiag {
