@@ -95,6 +95,8 @@ struct Instance {
         void* seg = nullptr;
         size_t seg_stride = 0;
         void* adj = nullptr;
+        size_t cp_bytes = 0, seg_bytes = 0, adj_bytes = 0;  // of the three allocations
+        int guards_K = 0;  // the segment layout (its K) whose guards are zero
         int filled = -1;  // segment whose per-step slots already hold its steps
     } rec;
 };
@@ -723,7 +725,7 @@ int step_instance(pwfa_lbm* h, Instance& in, const DiagOut* diag) {
 
 // ---------------------------------------------------------------- adjoint
 // One segment of a recording: the two population buffers the recomputed
-// forward steps ping-pong between, then E of each of its K states and B of
+// forward steps ping-pong between (the first step reads its checkpoint), then E of each of its K states and B of
 // its K + 1 states (each field array behind a zero guard), and the lattice
 // sums A_l ([4][N]) that each recomputed step stores for the reverse step.
 struct SegLayout {
@@ -771,23 +773,27 @@ StateRef state_at(const Instance& in, void* base, bool with_bn) {
     return r;
 }
 
-int copy_state(const Instance& in, const StateRef& dst, bool to_rec, cudaStream_t s) {
-    const size_t fb = (size_t)in.g.Np * kPop * storage_bytes(in.p.storage);
+int copy_fields(const Instance& in, const StateRef& dst, bool to_rec, cudaStream_t s) {
     const size_t vb = sizeof(float) * (size_t)in.g.N;
     if (to_rec) {
-        PWFA_CUDA(cudaMemcpyAsync(dst.f, in.f[in.fcur], fb, cudaMemcpyDeviceToDevice, s), "checkpoint copy");
         for (int c = 0; c < 3; ++c) {
             PWFA_CUDA(cudaMemcpyAsync(dst.E[c], in.E[c], vb, cudaMemcpyDeviceToDevice, s), "checkpoint copy");
             PWFA_CUDA(cudaMemcpyAsync(dst.B[c], in.B[in.bcur][c], vb, cudaMemcpyDeviceToDevice, s), "checkpoint copy");
         }
     } else {
-        PWFA_CUDA(cudaMemcpyAsync(in.f[in.fcur], dst.f, fb, cudaMemcpyDeviceToDevice, s), "restore copy");
         for (int c = 0; c < 3; ++c) {
             PWFA_CUDA(cudaMemcpyAsync(in.E[c], dst.E[c], vb, cudaMemcpyDeviceToDevice, s), "restore copy");
             PWFA_CUDA(cudaMemcpyAsync(in.B[in.bcur][c], dst.B[c], vb, cudaMemcpyDeviceToDevice, s), "restore copy");
         }
     }
     return PWFA_OK;
+}
+
+int copy_state(const Instance& in, const StateRef& dst, bool to_rec, cudaStream_t s) {
+    const size_t fb = (size_t)in.g.Np * kPop * storage_bytes(in.p.storage);
+    void* f = in.f[in.fcur];
+    PWFA_CUDA(cudaMemcpyAsync(to_rec ? dst.f : f, to_rec ? f : dst.f, fb, cudaMemcpyDeviceToDevice, s), "state copy");
+    return copy_fields(in, dst, to_rec, s);
 }
 
 // The built-in objective of the gradient calls (the witness loss): L =
@@ -853,17 +859,12 @@ int fill_segment(pwfa_lbm* h, Instance& in, int seg) {
     const int64_t N = in.g.N;
     const int64_t s0 = (int64_t)seg * r.K, s1 = std::min<int64_t>(r.T, s0 + r.K);
     const SegSlots S = seg_slots(in);
-    // restore the checkpoint into state 0 of the segment
-    {
-        StateRef cp = state_at(in, (char*)r.cp + r.cp_stride * seg, false);
-        const size_t fb = (size_t)in.g.Np * kPop * storage_bytes(in.p.storage);
-        PWFA_CUDA(cudaMemcpyAsync(S.pop(0), cp.f, fb, cudaMemcpyDeviceToDevice, s), "restore copy");
-        for (int c = 0; c < 3; ++c) {
-            PWFA_CUDA(cudaMemcpyAsync(S.E(0, c), cp.E[c], sizeof(float) * N, cudaMemcpyDeviceToDevice, s),
-                      "restore copy");
-            PWFA_CUDA(cudaMemcpyAsync(S.B(0, c), cp.B[c], sizeof(float) * N, cudaMemcpyDeviceToDevice, s),
-                      "restore copy");
-        }
+    // the checkpoint's fields into state 0 of the segment (behind its guards);
+    // its populations are read where they are
+    const StateRef cp = state_at(in, (char*)r.cp + r.cp_stride * seg, false);
+    for (int c = 0; c < 3; ++c) {
+        PWFA_CUDA(cudaMemcpyAsync(S.E(0, c), cp.E[c], sizeof(float) * N, cudaMemcpyDeviceToDevice, s), "restore copy");
+        PWFA_CUDA(cudaMemcpyAsync(S.B(0, c), cp.B[c], sizeof(float) * N, cudaMemcpyDeviceToDevice, s), "restore copy");
     }
     // recompute the segment's steps: populations ping-pong, E and B of
     // each state and the lattice sums of each step into their slots; Ampere
@@ -877,7 +878,7 @@ int fill_segment(pwfa_lbm* h, Instance& in, int seg) {
         StepArgs f = make_args(in);
         in.steps = keep_steps;
         const bool last = j + 1 == len;
-        f.fin = S.pop(j);
+        f.fin = j == 0 ? cp.f : S.pop(j);
         f.fout = last ? in.f[1 - in.fcur] : S.pop(j + 1);
         f.mom = S.mom(j);
         for (int c = 0; c < 3; ++c) {
@@ -927,49 +928,79 @@ int record_instance(pwfa_lbm* h, Instance& in, int32_t nsteps, int32_t ckpt_ever
     cudaStream_t s = h->stream;
     if (in.p.moving_window) return fail(PWFA_ERR_PARAM, "the adjoint does not support the moving window");
     if (in.p.driver != PWFA_DRIVER_RIGID) return fail(PWFA_ERR_PARAM, "the adjoint needs the rigid driver");
-    free_recording(in);
     auto& r = in.rec;
+    r.valid = false;
+    r.filled = -1;
     r.T = nsteps;
     r.K = ckpt_every > 0 ? ckpt_every : (int)std::ceil(std::sqrt((double)nsteps));
     if (r.K > nsteps) r.K = nsteps;
     r.ncp = (int)((nsteps + r.K - 1) / r.K);
     const size_t fb = fbytes_of(in), vb = vbytes_of(in);
     r.cp_stride = fb + 6 * vb;
-    const size_t seg_bytes = seg_layout(in, r.K).bytes();
+    const size_t cp_bytes = r.cp_stride * (r.ncp + 1);
+    const SegLayout L = seg_layout(in, r.K);
+    const size_t seg_bytes = L.bytes();
     const size_t adj_bytes = 2 * align_up((size_t)in.g.Np * kPop * sizeof(float)) + 22 * vb +
                              align_up(sizeof(double) * (260 + 3 * kGradSlots));
-    if (dev_alloc((void**)&r.cp, r.cp_stride * (r.ncp + 1)) != cudaSuccess ||
-        dev_alloc((void**)&r.seg, seg_bytes) != cudaSuccess ||
-        dev_alloc((void**)&r.adj, adj_bytes) != cudaSuccess) {
-        cudaGetLastError();
-        char buf[200];
-        std::snprintf(buf, sizeof buf, "recording needs %.2f GB (%d checkpoints + a segment of %d steps)",
-                      (r.cp_stride * (r.ncp + 1) + seg_bytes + adj_bytes) / 1e9, r.ncp + 1, r.K);
+    // The recording before leaves its allocations to this one unless they are
+    // too small, or more than twice too large (releasing and allocating the
+    // 18 GB of a 40-step recording of 256x128x128 took 12 of 35 ms).
+    auto fits = [](const void* p, size_t have, size_t need) { return p && have >= need && have / 2 <= need; };
+    if (!fits(r.cp, r.cp_bytes, cp_bytes) || !fits(r.seg, r.seg_bytes, seg_bytes) ||
+        !fits(r.adj, r.adj_bytes, adj_bytes)) {
+        const Instance::Recording want = r;
         free_recording(in);
-        return alloc_fail(buf);
+        if (dev_alloc((void**)&r.cp, cp_bytes) != cudaSuccess || dev_alloc((void**)&r.seg, seg_bytes) != cudaSuccess ||
+            dev_alloc((void**)&r.adj, adj_bytes) != cudaSuccess) {
+            cudaGetLastError();
+            char buf[200];
+            std::snprintf(buf, sizeof buf, "recording needs %.2f GB (%d checkpoints + a segment of %d steps)",
+                          (cp_bytes + seg_bytes + adj_bytes) / 1e9, want.ncp + 1, want.K);
+            free_recording(in);
+            return alloc_fail(buf);
+        }
+        r.T = want.T;
+        r.K = want.K;
+        r.ncp = want.ncp;
+        r.cp_stride = want.cp_stride;
+        r.cp_bytes = cp_bytes;
+        r.seg_bytes = seg_bytes;
+        r.adj_bytes = adj_bytes;
     }
-    // the guards in front of the segment's field slots stay zero
-    PWFA_CUDA(cudaMemsetAsync(r.seg, 0, seg_bytes, s), "cudaMemsetAsync");
+    // the guards in front of the segment's field slots: zero, and no step
+    // writes them
+    if (r.guards_K != r.K) {
+        r.guards_K = 0;
+        PWFA_CUDA(cudaMemset2DAsync((char*)r.seg + L.E(0, 0) - L.gb, L.gvb, 0, L.gb, (size_t)(6 * L.K + 3), s),
+                  "cudaMemset2DAsync");
+        r.guards_K = r.K;
+    }
+    // Each checkpoint's populations are the ones the run goes through there:
+    // the step before writes them into the checkpoint, in place of the
+    // instance's buffer, and the step after reads them from it (a copy would
+    // move 608 B/node for nothing).
+    void* const own[2] = {in.f[0], in.f[1]};
+    auto write_to = [&](int slot, int64_t n) {  // where state n goes
+        in.f[slot] = n % r.K ? own[slot] : (char*)r.cp + r.cp_stride * (n / r.K);
+    };
+    const int64_t s_last = (int64_t)(r.ncp - 1) * r.K;
+    write_to(0, 0);
     int rc = reset_instance(in, s);
-    if (rc) return rc;
     // the segments before the last one: ordinary steps with a checkpoint at
     // the start of each
-    const int64_t s_last = (int64_t)(r.ncp - 1) * r.K;
-    for (int64_t n = 0; n < s_last; ++n) {
-        if (n % r.K == 0) {
-            rc = copy_state(in, state_at(in, (char*)r.cp + r.cp_stride * (n / r.K), false), true, s);
-            if (rc) return rc;
-        }
+    for (int64_t n = 0; rc == PWFA_OK; ++n) {
+        if (n % r.K == 0) rc = copy_fields(in, state_at(in, (char*)r.cp + r.cp_stride * (n / r.K), false), true, s);
+        if (rc || n == s_last) break;
+        write_to(1 - in.fcur, n + 1);
         rc = step_instance(h, in);
-        if (rc) return rc;
     }
-    rc = copy_state(in, state_at(in, (char*)r.cp + r.cp_stride * (r.ncp - 1), false), true, s);
-    if (rc) return rc;
     // the last segment runs as the reverse sweep would recompute it, into
     // the segment slots, which the sweep then reverses first without a
     // recomputation (with one segment, ckpt_every >= nsteps, nothing is
     // recomputed at all)
-    rc = fill_segment(h, in, r.ncp - 1);
+    in.f[1 - in.fcur] = own[1 - in.fcur];
+    if (rc == PWFA_OK) rc = fill_segment(h, in, r.ncp - 1);
+    in.f[in.fcur] = own[in.fcur];
     if (rc) return rc;
     // the state at T: populations and E where the last step left them, B
     // from the segment's last slot
