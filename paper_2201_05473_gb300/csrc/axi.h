@@ -7,12 +7,16 @@
 // k nr + j (r fastest). Row 0 is the mirror image of row 1 (the axis lies
 // between them), rows 1..nr-2 hold the plasma, row nr-1 is the outer
 // boundary row. E_z at (z_{k+1/2}, r_j), E_r at (z_k, j dx), B_theta at
-// (z_{k+1/2}, j dx). Populations: [lattice][q][Np] planes (Np = N rounded up
-// to 32), the stored post-collision values that the next step pulls.
+// (z_{k+1/2}, j dx). Populations: the stored post-collision values that the
+// next step pulls, in chunks of 32 nodes that hold their 27 values one after
+// another: (l, q, node) at (node / 32) 27 32 + (9 l + q) 32 + node % 32. A
+// warp's 27 accesses fall in one or two 3.4 KB regions instead of 27 planes.
 #pragma once
 
 #include <cstdint>
 #include <cuda_runtime.h>
+
+#include "lbm_device.cuh"
 
 namespace pwfa {
 namespace axi {
@@ -22,7 +26,8 @@ constexpr int kL = 3;
 
 struct Args {
     int nz, nr;
-    int64_t N, Np;
+    int64_t N, Np;       // nodes; rounded up to whole chunks
+    FastDiv dnr;         // by nr
     const float* fin;    // streaming source of this step
     float* fout;         // post-collision populations written by this step
     float* Am;           // [3][N] node moments (exports)
@@ -48,6 +53,9 @@ struct Args {
 cudaError_t launch_moments(const Args& a, cudaStream_t s);
 cudaError_t launch_fluid(const Args& a, cudaStream_t s);
 cudaError_t launch_ampere(const Args& a, cudaStream_t s);
+// between the chunks and planes [3][9][N]
+cudaError_t launch_pack(const Args& a, const float* planes, float* f, cudaStream_t s);
+cudaError_t launch_unpack(const Args& a, const float* f, float* planes, cudaStream_t s);
 // plasma at rest: w_i n0 on lattice 0, zero on the momentum lattices
 cudaError_t launch_init(const Args& a, float* f, cudaStream_t s);
 // out[3][N] = n, beta_z, beta_r from the moments in a.Am

@@ -80,6 +80,7 @@ pwfa::axi::Args make_args(const pwfa_axi* h) {
     a.nr = p.nr;
     a.N = h->N;
     a.Np = h->Np;
+    a.dnr = pwfa::FastDiv((uint32_t)p.nr);
     a.fin = h->f[h->fcur];
     a.fout = h->f[1 - h->fcur];
     a.Am = h->Am;
@@ -132,18 +133,18 @@ int timed(pwfa_axi* h, int kind, const char* what, F&& launch) {
     return PWFA_OK;
 }
 
-// copies between a caller's [3][9][N] array (host or device) and the
-// [3][9][Np] population planes, one plane at a time
-int planes_to_user(pwfa_axi* h, const float* planes, float* user) {
-    for (int lq = 0; lq < 27; ++lq)
-        AXI_CUDA(cudaMemcpyAsync(user + (int64_t)lq * h->N, planes + (int64_t)lq * h->Np, sizeof(float) * h->N,
-                                 cudaMemcpyDefault, h->stream), "cudaMemcpyAsync");
+// copies between a caller's [3][9][N] array (host or device) and the chunked
+// populations, through the buffer the next step overwrites
+int source_to_user(pwfa_axi* h, float* user) {
+    float* planes = h->f[1 - h->fcur];
+    AXI_CUDA(pwfa::axi::launch_unpack(make_args(h), h->f[h->fcur], planes, h->stream), "unpack");
+    AXI_CUDA(cudaMemcpyAsync(user, planes, sizeof(float) * 27 * h->N, cudaMemcpyDefault, h->stream), "cudaMemcpyAsync");
     return PWFA_OK;
 }
-int user_to_planes(pwfa_axi* h, const float* user, float* planes) {
-    for (int lq = 0; lq < 27; ++lq)
-        AXI_CUDA(cudaMemcpyAsync(planes + (int64_t)lq * h->Np, user + (int64_t)lq * h->N, sizeof(float) * h->N,
-                                 cudaMemcpyDefault, h->stream), "cudaMemcpyAsync");
+int user_to_source(pwfa_axi* h, const float* user) {
+    float* planes = h->f[1 - h->fcur];
+    AXI_CUDA(cudaMemcpyAsync(planes, user, sizeof(float) * 27 * h->N, cudaMemcpyDefault, h->stream), "cudaMemcpyAsync");
+    AXI_CUDA(pwfa::axi::launch_pack(make_args(h), planes, h->f[h->fcur], h->stream), "pack");
     return PWFA_OK;
 }
 
@@ -245,7 +246,7 @@ int pwfa_axi_fields(pwfa_axi_t* h, float* out) {
 
 int pwfa_axi_get_source(pwfa_axi_t* h, float* fs) {
     if (!h || !fs) return set_error(PWFA_ERR_PARAM, "null argument");
-    int rc = planes_to_user(h, h->f[h->fcur], fs);
+    int rc = source_to_user(h, fs);
     if (rc) return rc;
     AXI_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     return PWFA_OK;
@@ -253,7 +254,7 @@ int pwfa_axi_get_source(pwfa_axi_t* h, float* fs) {
 
 int pwfa_axi_set_source(pwfa_axi_t* h, const float* fs) {
     if (!h || !fs) return set_error(PWFA_ERR_PARAM, "null argument");
-    int rc = user_to_planes(h, fs, h->f[h->fcur]);
+    int rc = user_to_source(h, fs);
     if (rc) return rc;
     AXI_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     return PWFA_OK;
