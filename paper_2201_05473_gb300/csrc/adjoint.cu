@@ -236,29 +236,24 @@ __device__ __forceinline__ int wall_candidates(int v, int n, int out[3]) {
     return m;
 }
 
-// Lattice-split form: a block of four warps takes 32 nodes of one x-row and
-// warp l owns lattice l. Each warp issues its lattice's 19 pulled populations
-// and 19 stored-population adjoints together (one memory round per node); the
-// lattice sums, the per-lattice reductions and the node-level adjoint (done
-// once, by warp 0) meet in shared memory.
-constexpr int kAdjThreads = 32 * kL;
-#ifndef PWFA_ADJ_MIN_BLOCKS
-#define PWFA_ADJ_MIN_BLOCKS 8
-#endif
-
-// The x = nx - 1 wall node of a row shares its block with the node it clamps
-// to (x = nx - 2) unless it opens a new block of 32.
-__host__ __device__ __forceinline__ bool xwall_split(int nx) { return (nx & 31) == 1; }
+// An x-wall node of an interior row is reversed with the row, in the warp of
+// the node it clamps to, unless that one opens the next warp or closes the one
+// before (never on rows of whole warps): then the shell pass takes it.
+__host__ __device__ __forceinline__ bool whole_warp_rows(const Grid& g) { return (g.nx & 31) == 0; }
+__device__ __forceinline__ bool xwall_alone(const Grid& g, int x, uint32_t node) {
+    return x == 0 ? (node & 31u) == 31u : (node & 31u) == 0u;
+}
 
 // Boundary nodes whose moment adjoints are produced by the shell pass: the
 // two z walls (nx ny each), then per interior plane the rows y = 0 and
-// y = ny - 1 (nx each) and, when the x = nx - 1 wall sits alone in its
-// block, the column x = nx - 1 of the interior rows (ny - 2). The other
-// x-wall nodes of interior rows are handled inside the interior pass, in
-// the block of the node they clamp to.
+// y = ny - 1 (nx each) and, where some may be alone, the columns x = 0 and
+// x = nx - 1 of the interior rows (ny - 2 each; those in a row's warp are
+// passed over).
+__host__ __device__ __forceinline__ uint32_t shell_ring(const Grid& g) {
+    return 2u * (uint32_t)g.nx + (whole_warp_rows(g) ? 0u : 2u * (uint32_t)(g.ny - 2));
+}
 __host__ __device__ __forceinline__ uint32_t shell_count(const Grid& g) {
-    const uint32_t ring = 2u * (uint32_t)g.nx + (xwall_split(g.nx) ? (uint32_t)(g.ny - 2) : 0u);
-    return 2u * (uint32_t)g.nx * (uint32_t)g.ny + (uint32_t)(g.nz - 2) * ring;
+    return 2u * (uint32_t)g.nx * (uint32_t)g.ny + (uint32_t)(g.nz - 2) * shell_ring(g);
 }
 
 __device__ __forceinline__ void shell_node(const Grid& g, uint32_t idx, int& x, int& y, int& z) {
@@ -271,7 +266,7 @@ __device__ __forceinline__ void shell_node(const Grid& g, uint32_t idx, int& x, 
         return;
     }
     idx -= 2u * P;
-    const uint32_t M = 2u * nx + (xwall_split(g.nx) ? (uint32_t)(g.ny - 2) : 0u);
+    const uint32_t M = shell_ring(g);
     const uint32_t k = idx / M;
     const uint32_t r = idx - k * M;
     z = 1 + (int)k;
@@ -279,99 +274,148 @@ __device__ __forceinline__ void shell_node(const Grid& g, uint32_t idx, int& x, 
         y = r < nx ? 0 : g.ny - 1;
         x = (int)(r < nx ? r : r - nx);
     } else {
-        x = g.nx - 1;
-        y = 1 + (int)(r - 2u * nx);
+        const uint32_t c = r - 2u * nx, rows = (uint32_t)(g.ny - 2);
+        x = c < rows ? 0 : g.nx - 1;
+        y = 1 + (int)(c < rows ? c : c - rows);
     }
 }
 
+// The sums over one lattice's 19 directions that the reverse collision needs:
+// G = sum w S, P = sum w S xi and W = sum w S xi (xi.u): per direction only
+// signed adds into the sums of its weight class (axis 1/18, diagonal 1/36),
+// weighted once at the end.
+struct AdjSums {
+    float G, P[3], W[3];
+};
+__device__ __forceinline__ AdjSums adj_sums(const float (&S)[kQ], const float u[3]) {
+    float G1 = 0.0f, G2 = 0.0f, P1[3] = {0.0f, 0.0f, 0.0f}, P2[3] = {0.0f, 0.0f, 0.0f};
+    float W1[3] = {0.0f, 0.0f, 0.0f}, W2[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int q = 1; q < kQ; ++q) {
+        float xu = 0.0f;
+        if (xi_x(q) > 0) xu += u[0]; else if (xi_x(q) < 0) xu -= u[0];
+        if (xi_y(q) > 0) xu += u[1]; else if (xi_y(q) < 0) xu -= u[1];
+        if (xi_z(q) > 0) xu += u[2]; else if (xi_z(q) < 0) xu -= u[2];
+        const float sx = S[q] * xu;
+        const bool diag = q > 6;
+        float& G = diag ? G2 : G1;
+        float* Pc = diag ? P2 : P1;
+        float* Wc = diag ? W2 : W1;
+        G += S[q];
+        if (xi_x(q) > 0) { Pc[0] += S[q]; Wc[0] += sx; } else if (xi_x(q) < 0) { Pc[0] -= S[q]; Wc[0] -= sx; }
+        if (xi_y(q) > 0) { Pc[1] += S[q]; Wc[1] += sx; } else if (xi_y(q) < 0) { Pc[1] -= S[q]; Wc[1] -= sx; }
+        if (xi_z(q) > 0) { Pc[2] += S[q]; Wc[2] += sx; } else if (xi_z(q) < 0) { Pc[2] -= S[q]; Wc[2] -= sx; }
+    }
+    const float wa = 1.0f / 18.0f, wd = 1.0f / 36.0f;
+    AdjSums v;
+    v.G = wq(0) * S[0] + wa * G1 + wd * G2;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        v.P[c] = wa * P1[c] + wd * P2[c];
+        v.W[c] = wa * W1[c] + wd * W2[c];
+    }
+    return v;
+}
+
+// One node per thread on runs of 128 consecutive nodes, as the forward fluid
+// step. Between reversed steps the adjoints f_bar of the pre-collision
+// populations are kept, each at its own node: the adjoint of a stored
+// population is S_bar_i(x) = f_bar_i(x + xi_i), so a thread gathers its 76
+// values like the forward pull and stores its own node's aligned. With them
+// come the node's lattice sums; each lattice's sums over its directions are
+// formed at once, and the node-level adjoint follows without a barrier.
 // SHELL: the shell nodes above (open grids), writing their moment adjoints
-// A_bar. Otherwise one block per 32 nodes of a row: interior nodes scatter
-// their population adjoints, boundary nodes zero the slots they pulled.
-template <int ST, int COLL, bool PER, bool SHELL>
-__global__ void __launch_bounds__(kAdjThreads, PWFA_ADJ_MIN_BLOCKS) adj_fluid_kernel(const AdjArgs a,
-                                                                                    uint32_t nshell) {
+// A_bar. Otherwise interior nodes write their f_bar and boundary nodes zero
+// (the forward step pulls nothing for them).
+//
+// Bounded by memory in the end (76 values in, 76 out, 22 and more of moments,
+// fields and adjoints: 696 B per node, 431 us at 256x128x128 of measured
+// copy bandwidth) and by registers on the way: 76 gathered values and the
+// sums want more than the 128 registers that leave 4 blocks on an SM, and
+// with fewer blocks too few loads are in flight. BGK, the one form that
+// needs the gathered values again at its end, parks those of lattices 2 and
+// 3 in shared memory meanwhile. Measured, both passes, BGK / regularized:
+// 256x128x128 517 / 515 us, 120x97x131 192 / 194, 64x32x32 19 / 19; before,
+// with a warp per lattice on blocks of 32 nodes of a row, sums passed through
+// shared memory and a scatter: 579 / 574, 253 / 249, 22 / 22. BGK without
+// parking 537; 3 blocks 556 / 565; 5 blocks 889 / 648 (spills); the fields'
+// loads before the gather 565; a scatter from one thread per node 588; every
+// x-wall node of a row that is no whole warps left to the shell pass
+// 250 / 239 at 120x97x131.
+template <int COLL, bool PER, bool SHELL>
+__global__ void __launch_bounds__(kLinearThreads, 4) adj_fluid_kernel(const AdjArgs a, const LinearMap m,
+                                                                      uint32_t nshell) {
     chain_begin();
-    using T = typename Codec<ST>::T;
-    __shared__ float sA[kL][32];     // lattice sums A_l
-    __shared__ float sG[kL][32];     // sum_i w_i S_bar_l,i
-    __shared__ float sU[kL][3][32];  // lattice l's share of u_bar
-    __shared__ float sN[4][3][32];   // node E, B sums at t_n and t_{n+1}, J_bar
-    __shared__ float sAb[kL][32];    // node-level part of A_bar; then x-wall A_bar
+    constexpr bool XIN = !PER && !SHELL;  // x-wall nodes along with the rows
+    constexpr bool PARK = COLL == 0 && !SHELL;
+    __shared__ float stash[PARK ? 2 * kQ : 1][kLinearThreads];
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(&stash[0][threadIdx.x]);
+    constexpr uint32_t kSRow = 4u * kLinearThreads;
     const StepArgs& s = a.f;
     const Grid& g = s.g;
-    const int l = (int)(threadIdx.x >> 5);
-    const int lane = (int)(threadIdx.x & 31);
-    int x, y, z;
+    int x = 0, y = 0, z = 0;
     bool live;
     if (SHELL) {
-        const uint32_t item = blockIdx.x * 32u + (uint32_t)lane;
+        const uint32_t item = blockIdx.x * kLinearThreads + threadIdx.x;
         live = item < nshell;
-        x = y = z = 0;
         if (live) shell_node(g, item, x, y, z);
     } else {
-        x = (int)blockIdx.x * 32 + lane;
-        y = (int)blockIdx.y;
-        z = (int)blockIdx.z;
-        live = x < g.nx;
+        live = m.node(g, x, y, z);
     }
     const uint32_t sxy = (uint32_t)g.nx * (uint32_t)g.ny;
     const uint32_t node = ((uint32_t)z * (uint32_t)g.ny + (uint32_t)y) * (uint32_t)g.nx + (uint32_t)x;
     const bool bnd = !PER && (x == 0 || y == 0 || z == 0 || x == g.nx - 1 || y == g.ny - 1 || z == g.nz - 1);
     const bool row_in = y >= 1 && y <= g.ny - 2 && z >= 1 && z <= g.nz - 2;
-    const bool xwall = !PER && !SHELL && live && row_in && (x == 0 || (x == g.nx - 1 && lane != 0));
+    const bool xside = x == 0 || x == g.nx - 1;
+    const bool xwall = XIN && live && row_in && xside && !xwall_alone(g, x, node);
+    if (SHELL && row_in && !xwall_alone(g, x, node)) live = false;
     const int64_t LS = lattice_stride(g);
-    const float* __restrict__ mom = s.mom;
-    const float* __restrict__ Sin = a.Sbar_in + l * LS;
-    float* __restrict__ Sout = a.Sbar_out + l * LS;
     if (!SHELL && live && bnd) {
-        // a boundary node's own pull slots are never read by the forward
-        // step: their adjoint is zero
+        // the forward step pulls nothing for a boundary node
 #pragma unroll
-        for (int q = 0; q < kQ; ++q) {
-            const int sx = x - xi_x(q), sy = y - xi_y(q), sz = z - xi_z(q);
-            if (!in_grid(g, sx, sy, sz)) continue;
-            const uint32_t so = PWFA_CHECK(
-                s.dbg, ((uint32_t)sz * (uint32_t)g.ny + (uint32_t)sy) * (uint32_t)g.nx + (uint32_t)sx, 0, g.Np, 7u);
-            Sout[pop_off(q, so)] = 0.0f;
-        }
+        for (int q = 0; q < kQ; ++q)
+#pragma unroll
+            for (int l = 0; l < kL; ++l) a.Fbar_out[l * LS + pop_off(q, node)] = 0.0f;
     }
     const bool act = live && (SHELL || !bnd || xwall);
-    // pulled node: the clamped interior node on open grids (Eq. 14)
-    int xs = x, ys = y, zs = z;
-    if (!PER) {
-        xs = min(max(x, 1), g.nx - 2);
-        ys = min(max(y, 1), g.ny - 2);
-        zs = min(max(z, 1), g.nz - 2);
-    }
-    const uint32_t nodec = ((uint32_t)zs * (uint32_t)g.ny + (uint32_t)ys) * (uint32_t)g.nx + (uint32_t)xs;
+    // (with XIN every lane stays for the exchange of the x-wall nodes)
+    if (!XIN && !act) return;
 
-    // ---- one memory round: this lattice's pulled populations and S_bar,
-    // plus one of the node's field sums (or J_bar) per warp
-    float S[kQ];
-    float Al = 0.0f;
-    const bool forced = (COLL != 2) && s.couple;
+    float S[kL][kQ], A[kL] = {1.0f, 0.0f, 0.0f, 0.0f};
     if (act) {
+        // S_bar_i(x) = f_bar_i(x + xi_i): the transposed pull. A neighbour
+        // outside an open grid is clamped to a boundary node, whose f_bar is
+        // zero as that slot's adjoint is.
+        const int ux = SHELL || XIN ? (x < g.nx - 1 ? 1 : 0) : 1, dx = SHELL || XIN ? (x > 0 ? 1 : 0) : 1;
+        const uint32_t uy = SHELL && y == g.ny - 1 ? 0u : (uint32_t)g.nx, dy = SHELL && y == 0 ? 0u : (uint32_t)g.nx;
+        const uint32_t uz = SHELL && z == g.nz - 1 ? 0u : sxy, dz = SHELL && z == 0 ? 0u : sxy;
 #pragma unroll
-        for (int q = 0; q < kQ; ++q) S[q] = __ldg(Sin + pop_off(q, node));
-        // the lattice sum of the node's pulled populations, as the forward
-        // step formed it (for a boundary node: of its clamped node's)
-        Al = __ldg(mom + (int64_t)l * g.N + node);
-        float v[3] = {0.0f, 0.0f, 0.0f};
-        if (l == 0) { if (forced) node_E<PER>(g, s.E, x, y, z, v, s.dbg); }
-        else if (l == 1) { if (forced) node_B_sum<PER>(g, s.Bc, x, y, z, v, s.dbg); }
-        else if (l == 2) { if (forced) node_B_sum<PER>(g, s.Bn, x, y, z, v, s.dbg); }
-        else { v[0] = a.Jbar[0][node]; v[1] = a.Jbar[1][node]; v[2] = a.Jbar[2][node]; }
+        for (int q = 0; q < kQ; ++q) {
+            uint32_t src = node;
+            if (PER) {
+                src = ((uint32_t)wrapi(z + xi_z(q), g.nz) * (uint32_t)g.ny + (uint32_t)wrapi(y + xi_y(q), g.ny)) *
+                          (uint32_t)g.nx + (uint32_t)wrapi(x + xi_x(q), g.nx);
+            } else {
+                if (xi_x(q) > 0) src += (uint32_t)ux; else if (xi_x(q) < 0) src -= (uint32_t)dx;
+                if (xi_y(q) > 0) src += uy; else if (xi_y(q) < 0) src -= dy;
+                if (xi_z(q) > 0) src += uz; else if (xi_z(q) < 0) src -= dz;
+            }
+            const uint32_t off = pop_off(q, PWFA_CHECK(s.dbg, src, 0, g.Np, 7u));
 #pragma unroll
-        for (int c = 0; c < 3; ++c) sN[l][c][lane] = v[c];
+            for (int l = 0; l < kL; ++l) S[l][q] = __ldg(a.Fbar_in + l * LS + off);
+        }
+        // the lattice sums of the node's pulled populations, as the forward
+        // step formed them (for a boundary node: of its clamped node's)
+#pragma unroll
+        for (int l = 0; l < kL; ++l) A[l] = __ldg(s.mom + (int64_t)l * g.N + node);
     } else {
 #pragma unroll
-        for (int q = 0; q < kQ; ++q) S[q] = 0.0f;
+        for (int l = 0; l < kL; ++l)
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) S[l][q] = 0.0f;
     }
-    sA[l][lane] = Al;
-    __syncthreads();
 
-    // ---- forward recompute of the node's velocity (every warp)
-    const float A[kL] = {sA[0][lane], sA[1][lane], sA[2][lane], sA[3][lane]};
+    // ---- the node's velocity
     const float n = A[0];
     const float nn = n > s.n_floor ? n : s.n_floor;
     const float inn = 1.0f / nn;
@@ -386,64 +430,51 @@ __global__ void __launch_bounds__(kAdjThreads, PWFA_ADJ_MIN_BLOCKS) adj_fluid_ke
     // stream-only, 1 for the regularized form and for boundary nodes
     const float wA = (COLL == 0 && !bnd) ? om : ((COLL == 2 && !bnd) ? 0.0f : 1.0f);
     const bool proj = COLL == 1 && !bnd;
+    const float base = 1.0f - 1.5f * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
 
-    // ---- this lattice's reductions over the 19 directions
-    // Gb = sum w S, P = sum w S xi, W = sum w S xi (xi.u) and
-    // sphi = sum w S phi_i / w_i = base Gb + 3 u.P + 4.5 u.W (since
-    // sum w S (xi.u)^2 = u.W): per direction only signed adds into the sums
-    // of its weight class (axis 1/18, diagonal 1/36), weighted once at the end.
-    float Gb, sphi, P[3], W[3];
-    {
-        float G1 = 0.0f, G2 = 0.0f, P1[3] = {0.0f, 0.0f, 0.0f}, P2[3] = {0.0f, 0.0f, 0.0f};
-        float W1[3] = {0.0f, 0.0f, 0.0f}, W2[3] = {0.0f, 0.0f, 0.0f};
+    // ---- each lattice's sums over the 19 directions: its own part of its
+    // moment adjoint, sum w S phi_i / w_i = base G + 3 u.P + 4.5 u.W (since
+    // sum w S (xi.u)^2 = u.W), and its share of u_bar, through
+    // phi_i = w_i (base + 3 xi.u + 4.5 (xi.u)^2) and the regularized
+    // projection's -k3 A_l P_l. Every lattice's share is rounded before it is
+    // added (no fused multiply-add), whichever thread forms it.
+    float Ab[kL], Gs[3], ub[3];
+    float mk[kL][3];  // (regularized: for the populations' adjoints)
 #pragma unroll
-        for (int q = 1; q < kQ; ++q) {
-            float xu = 0.0f;
-            if (xi_x(q) > 0) xu += u[0]; else if (xi_x(q) < 0) xu -= u[0];
-            if (xi_y(q) > 0) xu += u[1]; else if (xi_y(q) < 0) xu -= u[1];
-            if (xi_z(q) > 0) xu += u[2]; else if (xi_z(q) < 0) xu -= u[2];
-            const float sx = S[q] * xu;
-            const bool diag = q > 6;
-            float& G = diag ? G2 : G1;
-            float* Pc = diag ? P2 : P1;
-            float* Wc = diag ? W2 : W1;
-            G += S[q];
-            if (xi_x(q) > 0) { Pc[0] += S[q]; Wc[0] += sx; } else if (xi_x(q) < 0) { Pc[0] -= S[q]; Wc[0] -= sx; }
-            if (xi_y(q) > 0) { Pc[1] += S[q]; Wc[1] += sx; } else if (xi_y(q) < 0) { Pc[1] -= S[q]; Wc[1] -= sx; }
-            if (xi_z(q) > 0) { Pc[2] += S[q]; Wc[2] += sx; } else if (xi_z(q) < 0) { Pc[2] -= S[q]; Wc[2] -= sx; }
+    for (int l = 0; l < kL; ++l) {
+        const AdjSums v = adj_sums(S[l], u);
+        const float sphi = base * v.G + 3.0f * (u[0] * v.P[0] + u[1] * v.P[1] + u[2] * v.P[2]) +
+                           4.5f * (u[0] * v.W[0] + u[1] * v.W[1] + u[2] * v.W[2]);
+        Ab[l] = PER && COLL == 0 ? sphi : wA * sphi;
+        if (proj) Ab[l] -= k3 * (v.P[0] * u[0] + v.P[1] * u[1] + v.P[2] * u[2]);
+        if (l > 0) Gs[l - 1] = v.G;
+        if (PARK && l >= 2) {
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) stash_st(sbase + kSRow * ((l - 2) * kQ + q), S[l][q]);
         }
-        const float wa = 1.0f / 18.0f, wd = 1.0f / 36.0f;
-        Gb = wq(0) * S[0] + wa * G1 + wd * G2;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            P[c] = wa * P1[c] + wd * P2[c];
-            W[c] = wa * W1[c] + wd * W2[c];
+            float t = wA * A[l] * (3.0f * v.P[c] + 9.0f * v.W[c] - 3.0f * u[c] * v.G);
+            if (proj) t -= k3 * A[l] * v.P[c];
+            ub[c] = l == 0 ? t : __fadd_rn(ub[c], t);
+            if (COLL == 1) mk[l][c] = k3 * v.P[c];
         }
-        const float base = 1.0f - 1.5f * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-        sphi = base * Gb + 3.0f * (u[0] * P[0] + u[1] * P[1] + u[2] * P[2]) +
-               4.5f * (u[0] * W[0] + u[1] * W[1] + u[2] * W[2]);
     }
-    // u_bar share: d(A_l phi_i)/du through phi_i = w_i (base + 3 xi.u + 4.5 (xi.u)^2),
-    // plus the regularized projection's -k3 A_l P_l
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        float v = wA * Al * (3.0f * P[c] + 9.0f * W[c] - 3.0f * u[c] * Gb);
-        if (proj) v -= k3 * Al * P[c];
-        sU[l][c][lane] = v;
-    }
-    sG[l][lane] = Gb;
-    // this lattice's own part of its moment adjoint
-    float own = wA * sphi;
-    if (proj) own -= k3 * (P[0] * u[0] + P[1] * u[1] + P[2] * u[2]);
-    __syncthreads();
 
-    // ---- node-level reverse, once per node (warp 0)
-    if (l == 0 && act) {
+    // ---- node-level reverse
+    const bool forced = (COLL != 2) && s.couple;
+    if (act) {
         float e[3] = {0.0f, 0.0f, 0.0f}, b[3] = {0.0f, 0.0f, 0.0f}, F[3] = {0.0f, 0.0f, 0.0f};
+        const float Jb[3] = {__ldg(a.Jbar[0] + node), __ldg(a.Jbar[1] + node), __ldg(a.Jbar[2] + node)};
         if (forced) {
+            float bc[3], bn[3];
+            node_E<PER>(g, s.E, x, y, z, e, s.dbg);
+            node_B_sum<PER>(g, s.Bc, x, y, z, bc, s.dbg);
+            node_B_sum<PER>(g, s.Bn, x, y, z, bn, s.dbg);
+#pragma unroll
             for (int c = 0; c < 3; ++c) {
-                e[c] = sN[0][c][lane];
-                b[c] = 0.125f * (sN[1][c][lane] + sN[2][c][lane]);
+                b[c] = 0.125f * (bc[c] + bn[c]);
+                asm("" : "+f"(e[c]));  // the mean is rounded before it is used
             }
             F[0] = -n * (e[0] + beta[1] * b[2] - beta[2] * b[1]);
             F[1] = -n * (e[1] + beta[2] * b[0] - beta[0] * b[2]);
@@ -457,7 +488,6 @@ __global__ void __launch_bounds__(kAdjThreads, PWFA_ADJ_MIN_BLOCKS) adj_fluid_ke
         float nb, nnb = 0.0f;
         {
             // J = -n beta(p*)
-            const float Jb[3] = {sN[3][0][lane], sN[3][1][lane], sN[3][2][lane]};
             nb = -(Jb[0] * bs[0] + Jb[1] * bs[1] + Jb[2] * bs[2]);
             const float v[3] = {-n * Jb[0], -n * Jb[1], -n * Jb[2]};
             const float bv = bs[0] * v[0] + bs[1] * v[1] + bs[2] * v[2];
@@ -472,18 +502,18 @@ __global__ void __launch_bounds__(kAdjThreads, PWFA_ADJ_MIN_BLOCKS) adj_fluid_ke
         // source w_i F dt of lattices 1..3
         if (COLL != 2) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) Fb[c] += sG[c + 1][lane] * s.dt;
+            for (int c = 0; c < 3; ++c) Fb[c] += Gs[c] * s.dt;
         }
         float betab[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
-            betab[c] = s.lat * (sU[0][c][lane] + sU[1][c][lane] + sU[2][c][lane] + sU[3][c][lane]);
+        for (int c = 0; c < 3; ++c) betab[c] = s.lat * ub[c];
         float eb[3] = {0.0f, 0.0f, 0.0f}, bb[3] = {0.0f, 0.0f, 0.0f};
         if (forced) {
             // F = -n (e + beta x b)
             const float bxb[3] = {beta[1] * b[2] - beta[2] * b[1], beta[2] * b[0] - beta[0] * b[2],
                                   beta[0] * b[1] - beta[1] * b[0]};
             nb -= Fb[0] * (e[0] + bxb[0]) + Fb[1] * (e[1] + bxb[1]) + Fb[2] * (e[2] + bxb[2]);
+#pragma unroll
             for (int c = 0; c < 3; ++c) eb[c] = -n * Fb[c];
             // d/dbeta [Fb . (beta x b)] = b x Fb ;  d/db = Fb x beta
             betab[0] += -n * (b[1] * Fb[2] - b[2] * Fb[1]);
@@ -504,29 +534,41 @@ __global__ void __launch_bounds__(kAdjThreads, PWFA_ADJ_MIN_BLOCKS) adj_fluid_ke
             }
         }
         if (n > s.n_floor) nb += nnb;
-        sAb[0][lane] = nb;
-        sAb[1][lane] = Am[0];
-        sAb[2][lane] = Am[1];
-        sAb[3][lane] = Am[2];
+        // ---- the moment adjoints
+        // (on periodic BGK grids, where omega weights every node, the weight
+        // and the sum are one fused multiply-add)
+        auto plus = [&](float v, float own) { return PER && COLL == 0 ? __fmaf_rn(wA, own, v) : __fadd_rn(v, own); };
+        Ab[0] = plus(nb, Ab[0]);
+#pragma unroll
         for (int c = 0; c < 3; ++c) {
+            Ab[c + 1] = plus(Am[c], Ab[c + 1]);
             a.ebar[c][node] = eb[c];
             a.bbar[c][node] = bb[c];
         }
     }
-    __syncthreads();
-
-    // ---- this lattice's moment adjoint
-    float Ab = sAb[l][lane] + own;
     if (SHELL) {
-        if (act) a.Abnd[l][node] = Ab;
+#pragma unroll
+        for (int l = 0; l < kL; ++l) a.Abnd[l][node] = Ab[l];
         return;
     }
-    if (xwall) sAb[l][lane] = Ab;  // handed to the node it clamps to
-    __syncthreads();
-    if (!act || bnd) return;
     // Boundary nodes that gathered at this node add their A_bar to every
-    // population of the corresponding lattice: x-wall nodes of this row from
-    // shared memory, the shell nodes from the shell pass.
+    // population of the corresponding lattice: x-wall nodes in
+    // the warp from the neighbouring lanes, the others from the shell pass.
+    if (XIN) {
+        const unsigned all = 0xffffffffu;
+        const bool lo = x == 1 && (node & 31u) != 0u, hi = x == g.nx - 2 && (node & 31u) != 31u;
+        if (__any_sync(all, xwall)) {
+#pragma unroll
+            for (int l = 0; l < kL; ++l) {
+                const float up = __shfl_up_sync(all, Ab[l], 1), down = __shfl_down_sync(all, Ab[l], 1);
+                if (lo && row_in) Ab[l] += up;
+                if (hi && row_in) Ab[l] += down;
+            }
+        }
+        if (!act || bnd) return;
+    } else if (bnd) {
+        return;
+    }
     if (!PER && (x == 1 || y == 1 || z == 1 || x == g.nx - 2 || y == g.ny - 2 || z == g.nz - 2)) {
         int cx_[3], cy_[3], cz_[3];
         const int mx = wall_candidates(x, g.nx, cx_), my = wall_candidates(y, g.ny, cy_),
@@ -534,56 +576,28 @@ __global__ void __launch_bounds__(kAdjThreads, PWFA_ADJ_MIN_BLOCKS) adj_fluid_ke
         for (int iz = 0; iz < mz; ++iz)
             for (int iy = 0; iy < my; ++iy)
                 for (int ix = 0; ix < mx; ++ix) {
-                    if (ix == 0 && iy == 0 && iz == 0) continue;
-                    const int cx = cx_[ix];
-                    if (iy == 0 && iz == 0 && !(cx == g.nx - 1 && xwall_split(g.nx))) {
-                        Ab += sAb[l][cx == 0 ? lane - 1 : lane + 1];
-                    } else {
-                        const uint32_t bo =
-                            ((uint32_t)cz_[iz] * (uint32_t)g.ny + (uint32_t)cy_[iy]) * (uint32_t)g.nx + (uint32_t)cx;
-                        Ab += a.Abnd[l][bo];
-                    }
+                    if (iy == 0 && iz == 0 && (ix == 0 || !xwall_alone(g, cx_[ix], node - x + cx_[ix]))) continue;
+                    const uint32_t bo =
+                        ((uint32_t)cz_[iz] * (uint32_t)g.ny + (uint32_t)cy_[iy]) * (uint32_t)g.nx + (uint32_t)cx_[ix];
+#pragma unroll
+                    for (int l = 0; l < kL; ++l) Ab[l] += a.Abnd[l][bo];
                 }
     }
-    // transposed pull: f_i(x) = S_i(x - xi_i)  =>  S_bar_i(x - xi_i) = f_bar_i(x)
-    const float mk[3] = {k3 * P[0], k3 * P[1], k3 * P[2]};
-    auto fbar = [&](int q) {
-        float fb = Ab;
-        if (COLL == 0) fb += (1.0f - om) * S[q];
-        else if (COLL == 2) fb += S[q];
-        else fb += (float)xi_x(q) * mk[0] + (float)xi_y(q) * mk[1] + (float)xi_z(q) * mk[2];
+    // the adjoints of the node's pre-collision populations
+    auto fbar = [&](int l, int q) {
+        float fb = Ab[l];
+        if (COLL == 0) fb += (1.0f - om) * S[l][q];
+        else if (COLL == 2) fb += S[l][q];
+        else fb += (float)xi_x(q) * mk[l][0] + (float)xi_y(q) * mk[l][1] + (float)xi_z(q) * mk[l][2];
         return fb;
     };
-    if (!PER && (g.nx & 31) == 0) {
-        // nx a multiple of 32: x - xi_i lies xi_y nx + xi_z nx ny nodes (a
-        // whole number of 32-node chunks) from x - xi_x, and x -+ 1 crosses
-        // into the neighbouring chunk only at its first / last lane; so each
-        // slot is one of three per-node bases plus a per-direction shift
-        constexpr uint32_t kC = kQ * 32u;  // elements of one chunk
-        const uint32_t cy = (uint32_t)(g.nx >> 5) * kC, cz = (sxy >> 5) * kC;
-        const uint32_t l0 = nodec & 31u;
-        const uint32_t b0 = (nodec >> 5) * kC + l0;
-        const uint32_t bsrc_p = l0 == 31u ? b0 + kC - 31u : b0 + 1u;  // xi_x = -1: the source is x + 1
-        const uint32_t bsrc_m = l0 == 0u ? b0 - kC + 31u : b0 - 1u;   // xi_x = +1: the source is x - 1
+#pragma unroll
+    for (int l = 0; l < kL; ++l)
 #pragma unroll
         for (int q = 0; q < kQ; ++q) {
-            const uint32_t base = xi_x(q) > 0 ? bsrc_m : (xi_x(q) < 0 ? bsrc_p : b0);
-            uint32_t off = base + (uint32_t)q * 32u;
-            if (xi_y(q) > 0) off -= cy; else if (xi_y(q) < 0) off += cy;
-            if (xi_z(q) > 0) off -= cz; else if (xi_z(q) < 0) off += cz;
-            off = PWFA_CHECK(s.dbg, off, 0, (long long)kQ * g.Np, 7u);
-            Sout[off] = fbar(q);
+            if (PARK && l >= 2) S[l][q] = stash_ld(sbase + kSRow * ((l - 2) * kQ + q));
+            a.Fbar_out[l * LS + pop_off(q, node)] = fbar(l, q);
         }
-    } else {
-#pragma unroll
-        for (int q = 0; q < kQ; ++q) {
-            uint32_t src;
-            if (PER) src = (uint32_t)src_index<true>(g, xs, ys, zs, q);
-            else src = nodec - (uint32_t)(xi_x(q) + xi_y(q) * g.nx) - (uint32_t)xi_z(q) * sxy;
-            src = PWFA_CHECK(s.dbg, src, 0, g.Np, 7u);
-            Sout[pop_off(q, src)] = fbar(q);
-        }
-    }
 }
 
 // ------------------------------------------------------------------- R3
@@ -843,12 +857,12 @@ __global__ void __launch_bounds__(kRX * kRY, PWFA_ADJ_FE_MIN_BLOCKS) adj_faces_e
 }
 
 // ------------------------------------------------------------- profile
-// Initial stored populations S_0,i(y) = w_i n0 prof(r(y + xi_i)) with prof
-// piecewise linear in the profile values: accumulate S_bar w_i n0 times the
-// interpolation weights into the profile gradient.
+// Initial populations f_i(x) = w_i n0 prof(r(x)) of lattice 0 with prof
+// piecewise linear in the profile values: accumulate sum_i w_i f_bar_i n0
+// times the interpolation weights into the profile gradient.
 constexpr int kMaxProfile = 256;
 
-__global__ void __launch_bounds__(256) adj_profile_kernel(Grid g, const float* Sbar0, float n0, int np,
+__global__ void __launch_bounds__(256) adj_profile_kernel(Grid g, const float* Fbar0, float n0, int np,
                                                           double rmax, double dx, double* grad) {
     __shared__ double bins[kMaxProfile];
     for (int t = threadIdx.x; t < np; t += blockDim.x) bins[t] = 0.0;
@@ -863,27 +877,19 @@ __global__ void __launch_bounds__(256) adj_profile_kernel(Grid g, const float* S
         (void)z;
         const double xc = 0.5 * (g.nx - 1) * dx, yc = 0.5 * (g.ny - 1) * dx;
         const double h = np > 1 ? rmax / (np - 1) : 1.0;
-        for (int q = 0; q < kQ; ++q) {
-            const float sb = Sbar0[pop_off(q, (uint32_t)node)];
-            if (sb == 0.0f) continue;
-            int sx = x + xi_x(q), sy = y + xi_y(q);
-            if (g.periodic) { sx = wrapi(sx, g.nx); sy = wrapi(sy, g.ny); }
-            else { sx = min(max(sx, 1), g.nx - 2); sy = min(max(sy, 1), g.ny - 2); }
-            const double rx = sx * dx - xc, ry = sy * dx - yc;
+        double v = 0.0;
+        for (int q = 0; q < kQ; ++q) v += (double)Fbar0[pop_off(q, (uint32_t)node)] * wq(q);
+        v *= n0;
+        if (v != 0.0) {
+            const double rx = x * dx - xc, ry = y * dx - yc;
             const double r = sqrt(rx * rx + ry * ry);
-            const double v = (double)sb * wq(q) * n0;
-            if (np == 1 || r >= rmax) {
+            const int jj = np == 1 || r >= rmax ? np - 1 : (int)floor(r / h);
+            if (jj >= np - 1) {
                 atomicAdd(&bins[np - 1], v);
             } else {
-                const double tt = r / h;
-                int jj = (int)floor(tt);
-                if (jj >= np - 1) {
-                    atomicAdd(&bins[np - 1], v);
-                } else {
-                    const double fr = tt - jj;
-                    atomicAdd(&bins[jj], (1.0 - fr) * v);
-                    atomicAdd(&bins[jj + 1], fr * v);
-                }
+                const double fr = r / h - jj;
+                atomicAdd(&bins[jj], (1.0 - fr) * v);
+                atomicAdd(&bins[jj + 1], fr * v);
             }
         }
     }
@@ -894,27 +900,17 @@ __global__ void __launch_bounds__(256) adj_profile_kernel(Grid g, const float* S
 
 dim3 grid_of(const Grid& g, int bx, int by) { return dim3((g.nx + bx - 1) / bx, (g.ny + by - 1) / by, g.nz); }
 
-template <int ST, int COLL>
+template <int COLL>
 cudaError_t launch_adj_fluid_t(const AdjArgs& a, cudaStream_t s) {
     const Grid& g = a.f.g;
-    const dim3 rows((unsigned)(g.nx + 31) / 32, (unsigned)g.ny, (unsigned)g.nz);
-    if (g.periodic) {
-        return launch_chained(adj_fluid_kernel<ST, COLL, true, false>, rows, kAdjThreads, s, a, 0u);
-    }
+    const LinearMap m(g);
+    const unsigned runs = linear_blocks(g);
+    if (g.periodic) return launch_chained(adj_fluid_kernel<COLL, true, false>, runs, kLinearThreads, s, a, m, 0u);
     const uint32_t nb = shell_count(g);
-    cudaError_t e = launch_chained(adj_fluid_kernel<ST, COLL, false, true>, (nb + 31) / 32, kAdjThreads, s, a, nb);
+    cudaError_t e = launch_chained(adj_fluid_kernel<COLL, false, true>, (nb + kLinearThreads - 1) / kLinearThreads,
+                                   kLinearThreads, s, a, m, nb);
     if (e != cudaSuccess) return e;
-    return launch_chained(adj_fluid_kernel<ST, COLL, false, false>, rows, kAdjThreads, s, a, 0u);
-}
-
-template <int ST>
-cudaError_t launch_adj_fluid_s(const AdjArgs& a, int collision, cudaStream_t s) {
-    switch (collision) {
-        case 0: return launch_adj_fluid_t<ST, 0>(a, s);
-        case 1: return launch_adj_fluid_t<ST, 1>(a, s);
-        case 2: return launch_adj_fluid_t<ST, 2>(a, s);
-    }
-    return cudaErrorInvalidValue;
+    return launch_chained(adj_fluid_kernel<COLL, false, false>, runs, kLinearThreads, s, a, m, 0u);
 }
 
 }  // namespace
@@ -947,11 +943,12 @@ cudaError_t launch_adjoint_ampere(const AdjArgs& a0, cudaStream_t s) {
 }
 
 cudaError_t launch_adjoint_fluid(const AdjArgs& a0, int storage, int collision, cudaStream_t s) {
+    (void)storage;  // S_bar and the lattice sums are FP32 in every form
     const AdjArgs a = with_driver_factors(a0);
-    switch (storage) {
-        case 0: return launch_adj_fluid_s<0>(a, collision, s);
-        case 1: return launch_adj_fluid_s<1>(a, collision, s);
-        case 2: return launch_adj_fluid_s<2>(a, collision, s);
+    switch (collision) {
+        case 0: return launch_adj_fluid_t<0>(a, s);
+        case 1: return launch_adj_fluid_t<1>(a, s);
+        case 2: return launch_adj_fluid_t<2>(a, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -984,13 +981,13 @@ cudaError_t launch_adjoint_step(const AdjArgs& a, int storage, int collision, cu
     return e;
 }
 
-cudaError_t launch_adjoint_profile(const Grid& g, const float* Sbar, float n0, int n_profile, double rmax,
+cudaError_t launch_adjoint_profile(const Grid& g, const float* Fbar, float n0, int n_profile, double rmax,
                                    double dx, double* grad_profile, cudaStream_t s) {
     if (n_profile <= 0) return cudaSuccess;
     if (n_profile > kMaxProfile) return cudaErrorInvalidValue;
     const int threads = 256;
     const unsigned blocks = (unsigned)((g.N + threads - 1) / threads);
-    adj_profile_kernel<<<blocks, threads, 0, s>>>(g, Sbar, n0, n_profile, rmax, dx, grad_profile);
+    adj_profile_kernel<<<blocks, threads, 0, s>>>(g, Fbar, n0, n_profile, rmax, dx, grad_profile);
     return cudaGetLastError();
 }
 

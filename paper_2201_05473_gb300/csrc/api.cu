@@ -1039,7 +1039,7 @@ int adjoint_instance(pwfa_lbm* h, Instance& in, const float* seed_E, int32_t nst
     const size_t vb = vbytes_of(in);
     const size_t sb = align_up((size_t)in.g.Np * kPop * sizeof(float));
     char* p = static_cast<char*>(r.adj);
-    float* Sbar[2] = {(float*)p, (float*)(p + sb)};
+    float* Fbar[2] = {(float*)p, (float*)(p + sb)};
     p += 2 * sb;
     AdjArgs a{};
     float* Ebar[3];
@@ -1115,8 +1115,8 @@ int adjoint_instance(pwfa_lbm* h, Instance& in, const float* seed_E, int32_t nst
                 f.J[c] = nullptr;
             }
             a.f = f;
-            a.Sbar_in = Sbar[cur];
-            a.Sbar_out = Sbar[1 - cur];
+            a.Fbar_in = Fbar[cur];
+            a.Fbar_out = Fbar[1 - cur];
             int rc = timed_launch(h, PWFA_KERNEL_ADJ_FIELD, "adjoint ampere kernel",
                                   [&] { return launch_adjoint_ampere(a, s); });
             if (rc) return rc;
@@ -1131,7 +1131,7 @@ int adjoint_instance(pwfa_lbm* h, Instance& in, const float* seed_E, int32_t nst
         }
     }
     PWFA_CUDA(launch_adjoint_grad_finish(a.gslots, grad, s), "driver gradient");
-    PWFA_CUDA(launch_adjoint_profile(in.g, Sbar[cur], (float)in.p.n0, np, in.p.profile_rmax, in.p.dx, grad + 3, s),
+    PWFA_CUDA(launch_adjoint_profile(in.g, Fbar[cur], (float)in.p.n0, np, in.p.profile_rmax, in.p.dx, grad + 3, s),
               "profile gradient");
     PWFA_CUDA(cudaMemcpyAsync(host_grad, grad, sizeof(double) * (3 + np), cudaMemcpyDeviceToHost, s), "grad copy");
     int rc = copy_state(in, state_at(in, (char*)r.cp + r.cp_stride * r.ncp, false), false, s);

@@ -85,19 +85,8 @@ __device__ __forceinline__ void fluid_moments(const StepArgs& a, const float (&f
     }
 }
 
-// Shared-memory words of one thread's parked BGK values (lattices 2 and 3),
-// thread index fastest: a warp's 32 accesses of one value hit 32 banks. The
-// accesses are opaque to the compiler, so the parked registers are free
-// until the collision reads the words back.
+// Shared-memory words of one thread's parked BGK values (lattices 2 and 3).
 constexpr int kStashVals = 2 * kQ;
-__device__ __forceinline__ void stash_st(uint32_t a, float v) {
-    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v));
-}
-__device__ __forceinline__ float stash_ld(uint32_t a) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
-    return v;
-}
 
 // Everything after the moments: source, collision, stores, current. f holds
 // the pulled populations f^n(x) (of the clamped node when bnd; BGK and

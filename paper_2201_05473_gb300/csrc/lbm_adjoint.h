@@ -14,8 +14,8 @@ constexpr int kGradSlots = 1024;
 struct AdjArgs {
     StepArgs f;           // forward state of the reversed step: fin = S^{n-1},
                           // E = E^n, Bc = B(t_n), Bn = B(t_{n+1}), driver at t_{n+1}
-    const float* Sbar_in; // adjoint of the stored populations S^n, population layout (FP32)
-    float* Sbar_out;      // adjoint of S^{n-1}, population layout (FP32)
+    const float* Fbar_in; // adjoint of the pre-collision populations f^{n+1}, population layout (FP32)
+    float* Fbar_out;      // adjoint of f^n, population layout (FP32)
     float* Ebar[3];       // in: adjoint of E^{n+1}; out: adjoint of E^n
     float* Bbar[3];       // in: adjoint of B(t_{n+1}); out: adjoint of B(t_n)
     float* Bnp[3];        // scratch: adjoint of Bn at faces
@@ -41,9 +41,9 @@ cudaError_t launch_adjoint_step(const AdjArgs& a, int storage, int collision, cu
 // grad[0..2] = the sums of the driver-gradient slots.
 cudaError_t launch_adjoint_grad_finish(const double* gslots, double* grad, cudaStream_t s);
 
-// Profile gradient from the adjoint of the initial stored populations
-// (lattice 0 block of Sbar, population layout); n_profile <= 256.
-cudaError_t launch_adjoint_profile(const Grid& g, const float* Sbar, float n0, int n_profile, double rmax,
+// Profile gradient from the adjoint of the initial populations (lattice 0
+// block of Fbar, population layout); n_profile <= 256.
+cudaError_t launch_adjoint_profile(const Grid& g, const float* Fbar, float n0, int n_profile, double rmax,
                                    double dx, double* grad_profile, cudaStream_t s);
 
 }  // namespace pwfa

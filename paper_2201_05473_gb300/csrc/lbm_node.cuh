@@ -197,4 +197,16 @@ __device__ __forceinline__ void node_B_sum(const Grid& g, const float* const B[3
     }
 }
 
+// Values parked in shared memory, thread index fastest: a warp's 32 accesses
+// of one value hit 32 banks. The accesses are opaque to the compiler, so the
+// parked registers are free until the words are read back.
+__device__ __forceinline__ void stash_st(uint32_t a, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v));
+}
+__device__ __forceinline__ float stash_ld(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+
 }  // namespace pwfa
