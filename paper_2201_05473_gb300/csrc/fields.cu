@@ -78,21 +78,67 @@ __global__ void __launch_bounds__(kAFX * kAFY, PWFA_AF_MIN_BLOCKS)
     ampere_faraday_tile<PER>(a, out, blockIdx.x, blockIdx.y, blockIdx.z, a.zc);
 }
 
-// Blocks of four warps, each with its own nodes; eight blocks per SM (64
-// registers): six were slower at every size.
-template <int H>
-__global__ void __launch_bounds__(kARThreads, 8) ampere_faraday_rows_kernel(const StepArgs a, const FieldPair out) {
-    chain_begin();
-    const int n0 = (int)(blockIdx.x * (kARThreads / 32) + (threadIdx.x >> 5)) * kARNodes;
-    if (n0 >= a.g.nx * a.g.ny) return;
-    ampere_faraday_rows<H>(a, out, n0, blockIdx.y * H, a.zc);
+constexpr int64_t kPairNodes = (int64_t)256 << 10, kTileNodes = (int64_t)8 << 20;
+
+// Blocks of four warps, each with its own nodes; as many blocks per SM as
+// need no spills (V = 1: 64 registers, V = 2: 80).
+template <int V> constexpr int kARBlocks = V == 1 ? 8 : 6;
+
+// Blocks over a plane.
+unsigned rows_blocks(const Grid& g, int V) {
+    const int per = kARThreads / 32 * kARLanes * V;
+    return (unsigned)((g.nx * g.ny + per - 1) / per);
 }
 
-template <int H>
+template <int V, int H>
+__global__ void __launch_bounds__(kARThreads, kARBlocks<V>) ampere_faraday_rows_kernel(const StepArgs a,
+                                                                                       const FieldPair out) {
+    chain_begin();
+    const int n0 = (int)(blockIdx.x * (kARThreads / 32) + (threadIdx.x >> 5)) * kARLanes * V;
+    if (n0 >= a.g.nx * a.g.ny) return;
+    ampere_faraday_rows<V, H>(a, out, n0, blockIdx.y * H, a.zc);
+}
+
+template <int V, int H>
+cudaError_t launch_rows_h(const StepArgs& a, const FieldPair& out, cudaStream_t s) {
+    const dim3 grid(rows_blocks(a.g, V), (unsigned)((a.g.nz + H - 1) / H), 1);
+    return launch_chained(ampere_faraday_rows_kernel<V, H>, grid, kARThreads, s, a, out);
+}
+
+// Which fused kernel an open grid takes, and how many planes a warp marches:
+// more reuse more (B of the plane below, E of the plane above), fewer give
+// more warps. Field update per step on GB300, events included.
+//
+// Pairs of nodes (an even nx; every array starts on 256 bytes) from 256 Ki
+// nodes on: half the loads and address arithmetic per node, as many bytes in
+// flight with fewer warps. Against single nodes, and from 8 Mi nodes against
+// the tiles (15 loads a node, a barrier per plane), us: 512x256x256 398 -> 369
+// (tiles; 436 with single nodes), 256x128x128 64 -> 57, 192x96x96 33 -> 29,
+// 128x64x64 14.3 -> 12.6, 128x56x56 12.5 -> 11; 96x48x48 9.4 -> 10.2. Four
+// consecutive nodes per thread were slower (63 us at 256x128x128: 157
+// registers), and so were blocks of 256 or 384 threads and seven or eight
+// blocks per SM (spills). Planes: the fewest whose blocks the GPU holds at
+// once, up to four (128x64x64: 14.6, 13.1, 14.2 us with 2, 3, 4; 256x128x128
+// 87, 61.5, 59, 57 with 1 to 4, 61 with 8); eight from 8 Mi nodes on
+// (512x256x256: 377 with 4, 371).
+//
+// Single nodes otherwise: one plane up to 96 Ki nodes (64x32x32: 6.5 us, 8
+// with 2), two up to 640 Ki (96x48x48 8.7, 10.3 with 4), four above
+// (203x97x131: 46, 43). From 8 Mi nodes on the tiles take an odd nx
+// (512x256x255: 394 against 430).
 cudaError_t launch_rows(const StepArgs& a, const FieldPair& out, cudaStream_t s) {
-    const int per = kARThreads / 32 * kARNodes;
-    const dim3 grid((unsigned)((a.g.nx * a.g.ny + per - 1) / per), (unsigned)((a.g.nz + H - 1) / H), 1);
-    return launch_chained(ampere_faraday_rows_kernel<H>, grid, kARThreads, s, a, out);
+    if ((a.g.nx & 1) != 0 || a.g.N < kPairNodes) {
+        if (a.g.N < ((int64_t)96 << 10)) return launch_rows_h<1, 1>(a, out, s);
+        return a.g.N < ((int64_t)640 << 10) ? launch_rows_h<1, 2>(a, out, s) : launch_rows_h<1, 4>(a, out, s);
+    }
+    auto fits = [&](int h) {
+        return rows_blocks(a.g, 2) * (int64_t)((a.g.nz + h - 1) / h) <= 152 * kARBlocks<2>;
+    };
+    if (a.g.N >= kTileNodes) return launch_rows_h<2, 8>(a, out, s);
+    if (fits(1)) return launch_rows_h<2, 1>(a, out, s);
+    if (fits(2)) return launch_rows_h<2, 2>(a, out, s);
+    if (fits(3)) return launch_rows_h<2, 3>(a, out, s);
+    return launch_rows_h<2, 4>(a, out, s);
 }
 
 __global__ void __launch_bounds__(kBX * kBY) zero_walls_kernel(const StepArgs a) {
@@ -194,25 +240,9 @@ void fused_field_tiles(const Grid& g, int* tx, int* ty, int* tz) {
     *tz = (g.nz + kAFZ - 1) / kAFZ;
 }
 
-// Which fused kernel an open grid takes. The z-marching tiles move the least
-// (15 loads a node) and win where DRAM is the limit; below that their
-// blocks of 217 columns x 16 planes are too few or too long, and the rows
-// kernel, with no barrier and any number of planes per warp, is faster
-// (GB300, field update per step, events included, tiles against rows:
-// 512x256x256 396 against 426 us; 384x192x192 177 / 184; 256x128x128 66 / 64;
-// 192x96x96 40 / 32; 128x64x64 19.0 / 14.3; 64x32x32 12.9 / 7.0). More planes per
-// warp reuse more (B of the plane below, J_z of the one above), fewer give
-// more warps: one plane up to 96 Ki nodes (64x32x32: 7.0, 7.8, 8.7 us with 1,
-// 2, 4), two up to 1 Mi (96x48x48: 10.4, 8.7, 10.3), four above
-// (203x97x131: 55, 46, 44).
-constexpr int64_t kRows2Nodes = (int64_t)96 << 10, kRows4Nodes = (int64_t)1 << 20, kTileNodes = (int64_t)8 << 20;
-
 cudaError_t launch_ampere_faraday(const StepArgs& a, const FieldPair& out, cudaStream_t s) {
     if (a.Jb[0]) return cudaErrorInvalidValue;  // the PIC deposit is cleared by the plain Ampere kernel
-    if (!a.g.periodic && a.g.N < kTileNodes) {
-        if (a.g.N < kRows2Nodes) return launch_rows<1>(a, out, s);
-        return a.g.N < kRows4Nodes ? launch_rows<2>(a, out, s) : launch_rows<4>(a, out, s);
-    }
+    if (!a.g.periodic && (a.g.N < kTileNodes || (a.g.nx & 1) == 0)) return launch_rows(a, out, s);
     const dim3 block(kAFX, kAFY, 1);
     const dim3 grid((a.g.nx + kAFX - 2) / (kAFX - 1), (a.g.ny + kAFY - 2) / (kAFY - 1), (a.g.nz + kAFZ - 1) / kAFZ);
     return launch_chained(a.g.periodic ? ampere_faraday_kernel<true> : ampere_faraday_kernel<false>, grid, block, s, a,
