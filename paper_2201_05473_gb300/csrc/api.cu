@@ -515,10 +515,8 @@ int batch_build(pwfa_lbm* h) {
         e.ntiles = (in.g.N + kBatchTile - 1) / kBatchTile;
         e.tile_begin = ntiles;
         ntiles += (e.ntiles + kBatchGroup - 1) / kBatchGroup;
-        int fz = 0;
-        fused_field_tiles(in.g, &e.ftiles_x, &e.ftiles_y, &fz);
         e.ftile_begin = nftiles;
-        nftiles += (int64_t)e.ftiles_x * e.ftiles_y * fz;
+        nftiles += batch_field_tiles(in.g, e);
         e.z0 = in.p.z0;
         e.dt = in.p.dt;
         e.step = h->d_steps;  // set below, once the counters exist

@@ -2,13 +2,14 @@
 // together, one launch per phase for all of them, two steps replayed from a
 // captured CUDA graph. Each phase is one grid over the concatenated tiles of
 // every instance (per-node phases: groups of tiles of 128 consecutive nodes;
-// fused field step: the z-marching tiles of fields_fused.cuh); a 16-bit
-// table maps each block to its instance. The hardware block
+// fused field step: groups of four warps of fields_rows.cuh, on periodic grids
+// the z-marching tiles of fields_fused.cuh); a 16-bit table maps each block to its instance. The hardware block
 // scheduler hands the tiles out in order, so the tiles in flight form one
 // short window of the list and the z +- 1 planes a pull reads are still in
 // L2. No block waits on another.
 #include "lbm_batch.h"
 #include "fields_fused.cuh"
+#include "fields_rows.cuh"
 #include "fluid_node.cuh"
 
 namespace pwfa {
@@ -97,6 +98,45 @@ __global__ void __launch_bounds__(kAFX * kAFY, PWFA_AF_MIN_BLOCKS)
     ampere_faraday_tile<PER>(sa, so, r - tby * e.ftiles_x, tby, tbz, s_zc);
 }
 
+// The same on open grids, on rows of nodes: a block takes four consecutive
+// warps of its instance, counted plane by plane over slabs of H planes. The
+// tiles, whose 31 x 7 columns fit few of a batch's grids, and the same body as
+// a single launch's (two nodes per thread where nx is even). Whole steps on
+// GB300, tiles / rows, us: 32 instances of 64x32x32 to 256x128x128 6133 /
+// 5999 (with H = 2, 4, 6: 6134, 6047, 6033), 256 of 32x16x16 278 / 257.5
+// (H = 8: 262, too few warps for one more wave), one less in x and y 6046 /
+// 6006 and 282 / 265. Five or seven blocks per SM 6004 and 6057.
+__host__ __device__ __forceinline__ int rows_vector(const Grid& g) { return (g.nx & 1) == 0 ? 2 : 1; }
+__host__ __device__ __forceinline__ int rows_planes(const Grid& g) { return g.N < ((int64_t)32 << 10) ? 4 : 8; }
+
+__global__ void __launch_bounds__(kARThreads, 6)
+    batch_rows_kernel(const BatchEntry* __restrict__ ent, const uint16_t* __restrict__ ftile_inst, int parity) {
+    __shared__ StepArgs sa;
+    __shared__ FieldPair so;
+    __shared__ float s_zc;
+    const int tid = threadIdx.x;
+    const int inst = __ldg(ftile_inst + blockIdx.x);
+    const BatchEntry& e = ent[inst];
+    copy_words<kARThreads>(&sa, &e.args[parity], sizeof(StepArgs), tid);
+    copy_words<kARThreads>(&so, &e.out[parity], sizeof(FieldPair), tid);
+    const int64_t local = (int64_t)blockIdx.x - e.ftile_begin;
+    if (tid == 0) s_zc = driver_centre(e, parity, local == 0);
+    const int per_plane = e.ftiles_x;
+    __syncthreads();
+    const int V = rows_vector(sa.g), H = rows_planes(sa.g);
+    const int w = (int)local * (kARThreads / 32) + (tid >> 5);
+    const int slab = w / per_plane;
+    const int k0 = slab * H, n0 = (w - slab * per_plane) * kARLanes * V;
+    if (k0 >= sa.g.nz) return;
+    if (V == 2) {
+        if (H == 8) ampere_faraday_rows<2, 8>(sa, so, n0, k0, s_zc);
+        else ampere_faraday_rows<2, 4>(sa, so, n0, k0, s_zc);
+    } else {
+        if (H == 8) ampere_faraday_rows<1, 8>(sa, so, n0, k0, s_zc);
+        else ampere_faraday_rows<1, 4>(sa, so, n0, k0, s_zc);
+    }
+}
+
 template <int ST, int COLL, bool PER>
 cudaError_t launch_phase(const BatchLaunch& b, int phase, int parity, cudaStream_t s) {
     const unsigned nt = (unsigned)b.ntiles;
@@ -105,7 +145,11 @@ cudaError_t launch_phase(const BatchLaunch& b, int phase, int parity, cudaStream
         case 1: batch_node_kernel<ST, COLL, PER, 1><<<nt, kBatchTile, 0, s>>>(b.entries, b.tile_inst, parity); break;
         case 2: batch_node_kernel<ST, COLL, PER, 2><<<nt, kBatchTile, 0, s>>>(b.entries, b.tile_inst, parity); break;
         case 3:
-            batch_fields_kernel<PER><<<(unsigned)b.nftiles, dim3(kAFX, kAFY, 1), 0, s>>>(b.entries, b.ftile_inst, parity);
+            if (PER)
+                batch_fields_kernel<PER><<<(unsigned)b.nftiles, dim3(kAFX, kAFY, 1), 0, s>>>(b.entries, b.ftile_inst,
+                                                                                             parity);
+            else
+                batch_rows_kernel<<<(unsigned)b.nftiles, kARThreads, 0, s>>>(b.entries, b.ftile_inst, parity);
             break;
         default: return cudaErrorInvalidValue;
     }
@@ -129,6 +173,19 @@ cudaError_t launch_phase_c(const BatchLaunch& b, int phase, int parity, int coll
 }
 
 }  // namespace
+
+int64_t batch_field_tiles(const Grid& g, BatchEntry& e) {
+    if (g.periodic) {
+        int tz = 0;
+        fused_field_tiles(g, &e.ftiles_x, &e.ftiles_y, &tz);
+        return (int64_t)e.ftiles_x * e.ftiles_y * tz;
+    }
+    const int nodes = kARLanes * rows_vector(g), H = rows_planes(g);
+    e.ftiles_x = (g.nx * g.ny + nodes - 1) / nodes;
+    e.ftiles_y = 1;
+    const int64_t warps = (int64_t)e.ftiles_x * ((g.nz + H - 1) / H);
+    return (warps + kARThreads / 32 - 1) / (kARThreads / 32);
+}
 
 cudaError_t launch_batch_phase(const BatchLaunch& b, int phase, int parity, int storage, int collision,
                                bool periodic, cudaStream_t s) {

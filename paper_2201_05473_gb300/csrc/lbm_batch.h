@@ -21,8 +21,9 @@ struct BatchEntry {
     FieldPair out[2];     // the fused field step's outputs for the two parities
     int64_t tile_begin;   // first block (group of kBatchGroup fluid tiles) of the instance
     int64_t ntiles;       // fluid tiles of the instance
-    int64_t ftile_begin;  // first fused-field tile
-    int ftiles_x, ftiles_y;  // fused-field tiles per z-slab
+    int64_t ftile_begin;  // first fused-field tile (block)
+    int ftiles_x, ftiles_y;  // periodic: fused-field tiles per z-slab; open:
+                             // warps per plane, 1
     double z0, dt;        // driver centre at t = 0 and time step
     int64_t* step;        // two device step counters: the step index n of the
                           // step that the launches of parity p take is
@@ -38,6 +39,9 @@ struct BatchLaunch {
     int ninst;
     int64_t ntiles, nftiles;           // blocks of the per-node phases, fused-field tiles
 };
+
+// The instance's fused-field blocks; sets e.ftiles_x and e.ftiles_y.
+int64_t batch_field_tiles(const Grid& g, BatchEntry& e);
 
 // Phases of one batched step: 0 Faraday, 1 fluid, 2 Ampere (per-node, on
 // the fluid tiles), 3 Ampere fused with the next step's Faraday (on the
