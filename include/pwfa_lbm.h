@@ -149,8 +149,9 @@ int pwfa_lbm_step(pwfa_lbm_t* h, int32_t nsteps);
  *
  * pwfa_lbm_record resets the instance to its initial condition (t = 0) and
  * advances it nsteps, keeping a checkpoint of the full state every
- * ckpt_every steps (0 selects ceil(sqrt(nsteps))) plus the final state. The
- * instance is left at step nsteps. Device memory: (nsteps/ckpt_every + 1)
+ * ckpt_every steps (0 selects ceil(sqrt(nsteps)), or nsteps, one segment,
+ * where that takes no more memory: up to some 65 steps in FP32, 20 in 16-bit
+ * storage) plus the final state. The instance is left at step nsteps. Device memory: (nsteps/ckpt_every + 1)
  * states of 76 N populations + 6 N field values; one segment of K =
  * ckpt_every recomputed steps (two population buffers, the E and B of its
  * states, 6 (K + 1) N values, and the four lattice sums of each step, 4 K N:
@@ -174,8 +175,8 @@ int pwfa_lbm_record(pwfa_lbm_t* h, int32_t instance, int32_t nsteps, int32_t ckp
  *           instance already holds a recording of T steps (with ckpt_every
  *           checkpoints when ckpt_every > 0); 0: use the existing recording
  *           (PWFA_ERR_STATE if there is none).
- *   ckpt_every  checkpoint interval of a new recording; 0 selects
- *           ceil(sqrt(T)).
+ *   ckpt_every  checkpoint interval of a new recording; 0 selects one as
+ *           pwfa_lbm_record does.
  * Each segment is recomputed from its checkpoint, then reversed: transposed
  * Ampere (with the driver's parameter derivatives), transposed fluid step
  * (J = -n beta(p*), collision, equilibrium, Lorentz source, beta(p), the

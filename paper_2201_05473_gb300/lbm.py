@@ -353,7 +353,9 @@ class Simulation:
         _check(self._lib.pwfa_lbm_autotune(self._h, reps))
 
     def record(self, nsteps: int, ckpt_every: int = 0, instance: int = 0):
-        """Reset to t = 0 and run nsteps keeping checkpoints for the adjoint."""
+        """Reset to t = 0 and run nsteps keeping checkpoints for the adjoint
+        (ckpt_every = 0: every ceil(sqrt(nsteps)) steps, or one segment and
+        nothing to recompute where that takes no more memory)."""
         _check(self._lib.pwfa_lbm_record(self._h, instance, int(nsteps), int(ckpt_every)))
 
     def adjoint_step(self, seed_E=None, nsteps: int = 0, ckpt_every: int = 0, instance: int = 0) -> np.ndarray:
