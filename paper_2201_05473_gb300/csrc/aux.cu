@@ -1,6 +1,7 @@
 // Set-up, state exchange and diagnostics kernels (not on the per-step path).
 #include "lbm_kernels.h"
 #include "lbm_node.cuh"
+#include "launch.cuh"
 
 namespace pwfa {
 
@@ -198,82 +199,136 @@ __global__ void linecut_kernel(const StepArgs a, double xr, float* out) {
 }
 
 // ---------------------------------------------------------------- diagnostics
+// FP64 arithmetic is scarce on this part (two lanes an SM and clock, and
+// every conversion takes one): what bounds these kernels. So only the sums
+// are formed in FP64; minimum and count stay in FP32 and integers, which
+// hold them exactly, the maximum of |beta|^2 is kept by its bits (those of
+// non-negative doubles order as integers) and its root, which is monotonic,
+// is taken once per block.
 struct Diag {
-    double sn, s1, s2, s3, en, mn, mb, bad;
+    double s[5];      // sums of n, n p_x, n p_y, n p_z, field energy
+    float mn;         // min n (infinity: no finite one)
+    long long mb;     // bits of max |beta|^2 (or of max |beta|)
+    int bad;          // non-finite nodes
 };
+__device__ __forceinline__ Diag diag_none() { return Diag{{0, 0, 0, 0, 0}, __int_as_float(0x7f800000), 0, 0}; }
 
-__device__ __forceinline__ void diag_combine(Diag& a, const Diag& b) {
-    a.sn += b.sn; a.s1 += b.s1; a.s2 += b.s2; a.s3 += b.s3; a.en += b.en;
-    a.mn = fmin(a.mn, b.mn); a.mb = fmax(a.mb, b.mb); a.bad += b.bad;
-}
-
-__device__ __forceinline__ Diag diag_shfl(const Diag& d, int off) {
-    Diag r;
-    r.sn = __shfl_down_sync(0xffffffffu, d.sn, off);
-    r.s1 = __shfl_down_sync(0xffffffffu, d.s1, off);
-    r.s2 = __shfl_down_sync(0xffffffffu, d.s2, off);
-    r.s3 = __shfl_down_sync(0xffffffffu, d.s3, off);
-    r.en = __shfl_down_sync(0xffffffffu, d.en, off);
-    r.mn = __shfl_down_sync(0xffffffffu, d.mn, off);
-    r.mb = __shfl_down_sync(0xffffffffu, d.mb, off);
-    r.bad = __shfl_down_sync(0xffffffffu, d.bad, off);
-    return r;
-}
-
-// Block reduction (warp shuffles, then one warp over the warp results).
-__device__ void diag_block_reduce(Diag d, double* dst) {
-    __shared__ Diag sh[kDiagThreads / 32];
-    for (int off = 16; off > 0; off >>= 1) diag_combine(d, diag_shfl(d, off));
+// Block reduction to one record of 8 doubles: sums over a warp by recursive
+// halving (as diag8_warp of the fluid kernel: 9 adds a lane instead of 40),
+// then 8 threads over the warps. ROOT: mb holds squares.
+template <bool ROOT>
+__device__ void diag_block_reduce(const Diag& d, double* dst) {
+    constexpr int W = kDiagThreads / 32;
+    __shared__ double shs[W][8];
+    __shared__ float shm[W];
+    __shared__ long long shb[W];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) sh[warp] = d;
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+    const double v[8] = {d.s[0], d.s[1], d.s[2], d.s[3], d.s[4], (double)d.bad, 0.0, 0.0};
+    double w[4], u[2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double keep = b4 ? v[k + 4] : v[k], send = b4 ? v[k] : v[k + 4];
+        w[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const double keep = b3 ? w[k + 2] : w[k], send = b3 ? w[k] : w[k + 2];
+        u[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+    }
+    double t = (b2 ? u[1] : u[0]) + __shfl_xor_sync(0xffffffffu, b2 ? u[0] : u[1], 4);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    float mn = d.mn;
+    long long mb = d.mb;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
+        const long long o = __shfl_xor_sync(0xffffffffu, mb, off);
+        mb = o > mb ? o : mb;
+    }
+    if ((lane & 3) == 0) shs[warp][lane >> 2] = t;
+    if (lane == 0) {
+        shm[warp] = mn;
+        shb[warp] = mb;
+    }
     __syncthreads();
-    if (warp == 0) {
-        d = lane < kDiagThreads / 32 ? sh[lane] : Diag{0, 0, 0, 0, 0, 1e300, 0, 0};
-        for (int off = 16; off > 0; off >>= 1) diag_combine(d, diag_shfl(d, off));
-        if (lane == 0) {
-            dst[0] = d.sn; dst[1] = d.s1; dst[2] = d.s2; dst[3] = d.s3;
-            dst[4] = d.en; dst[5] = d.mn; dst[6] = d.mb; dst[7] = d.bad;
-        }
+    if (threadIdx.x < 6) {
+        double r = 0.0;
+        for (int k = 0; k < W; ++k) r += shs[k][threadIdx.x];
+        dst[threadIdx.x == 5 ? 7 : threadIdx.x] = r;
+    } else if (threadIdx.x == 6) {
+        for (int k = 0; k < W; ++k) mn = fminf(mn, shm[k]);
+        dst[5] = isinf(mn) && mn > 0.0f ? 1e300 : (double)mn;
+    } else if (threadIdx.x == 32) {
+        for (int k = 0; k < W; ++k) mb = shb[k] > mb ? shb[k] : mb;
+        dst[6] = ROOT ? sqrt(__longlong_as_double(mb)) : __longlong_as_double(mb);
     }
 }
 
-// Grid-stride over nodes; one partial record of 8 doubles per block.
+// Runs of kDiagThreads nodes, run after run; one partial record of 8 doubles
+// per block. |beta|^2 is formed in FP64 only where its FP32 value is not
+// below the largest one of the warp's runs so far (by more than the FP32 error,
+// 1e-6 of it or 1e-37), and where it is not zero. Whole diagnostics call at
+// 256x128x128 FP32 on GB300: 467 -> 241 us, some 25 of them the copy to the
+// host (203 at the copy bandwidth); before, minimum, maximum and a root per
+// node in FP64.
 template <int ST, bool PER>
-__global__ void __launch_bounds__(kDiagThreads) diag_kernel(const StepArgs a, double dxcube, double* partials) {
+__global__ void __launch_bounds__(kDiagThreads, 2)
+    diag_kernel(const StepArgs a, const FastDiv nxy, const FastDiv nx, double dxcube, double* partials) {
+    chain_begin();
     using T = typename Codec<ST>::T;
     const Grid& g = a.g;
-    Diag d{0, 0, 0, 0, 0, 1e300, 0, 0};
-    for (int64_t node = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; node < g.N;
-         node += (int64_t)gridDim.x * blockDim.x) {
-        int x, y, z;
-        node_xyz(g, node, x, y, z);
-        float f[kL][kQ];
-        bool bnd;
-        gather<ST, PER>(g, static_cast<const T*>(a.fin), a.n0, x, y, z, f, bnd, 0u, a.dbg);
-        float A[kL], inn, beta[3];
-        node_moments(f, a.n_floor, A, inn, beta);
-        const bool fin = isfinite(A[0]) && isfinite(A[1]) && isfinite(A[2]) && isfinite(A[3]);
-        d.bad += fin ? 0.0 : 1.0;
-        d.sn += A[0]; d.s1 += A[1]; d.s2 += A[2]; d.s3 += A[3];
-        d.mn = fmin(d.mn, (double)A[0]);
-        d.mb = fmax(d.mb, sqrt((double)beta[0] * beta[0] + (double)beta[1] * beta[1] + (double)beta[2] * beta[2]));
-        double e2 = 0.0;
-        for (int c = 0; c < 3; ++c) {
-            const double ev = a.E[c][node], bv = a.Bc[c][node];
-            e2 += ev * ev + bv * bv;
+    Diag d = diag_none();
+    float top = 0.0f;  // the warp's largest FP32 |beta|^2
+    for (uint32_t run = blockIdx.x; (int64_t)run * kDiagThreads < g.N; run += gridDim.x) {
+        const uint32_t node = run * kDiagThreads + threadIdx.x;
+        float b2 = 0.0f, beta[3] = {0.0f, 0.0f, 0.0f};
+        if (node < (uint32_t)g.N) {
+            const uint32_t k = nxy.div(node), r = node - k * nxy.d, j = nx.div(r);
+            float f[kL][kQ];
+            bool bnd;
+            gather<ST, PER>(g, static_cast<const T*>(a.fin), a.n0, (int)(r - j * nx.d), (int)j, (int)k, f, bnd, 0u,
+                            a.dbg);
+            float e[6];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                e[c] = __ldg(a.E[c] + node);
+                e[3 + c] = __ldg(a.Bc[c] + node);
+            }
+            float A[kL], inn;
+            node_moments(f, a.n_floor, A, inn, beta);
+            const bool fin = isfinite(A[0]) && isfinite(A[1]) && isfinite(A[2]) && isfinite(A[3]);
+            d.bad += fin ? 0 : 1;
+#pragma unroll
+            for (int l = 0; l < kL; ++l) d.s[l] += A[l];
+            d.mn = fminf(d.mn, A[0]);
+            b2 = beta[0] * beta[0] + beta[1] * beta[1] + beta[2] * beta[2];
+#pragma unroll
+            for (int c = 0; c < 6; ++c) d.s[4] += (double)e[c] * e[c];
         }
-        d.en += 0.5 * e2 * dxcube;
+        if ((beta[0] != 0.0f || beta[1] != 0.0f || beta[2] != 0.0f) && b2 >= top * 0.999999f - 1e-37f) {
+            const double v = (double)beta[0] * beta[0] + (double)beta[1] * beta[1] + (double)beta[2] * beta[2];
+            d.mb = max(d.mb, __double_as_longlong(v));
+        }
+        top = __uint_as_float(
+            __reduce_max_sync(0xffffffffu, __float_as_uint(b2 > top ? b2 : top)));
     }
-    diag_block_reduce(d, partials + 8 * (int64_t)blockIdx.x);
+    d.s[4] *= 0.5 * dxcube;
+    diag_block_reduce<true>(d, partials + 8 * (int64_t)blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kDiagThreads) diag_finish_kernel(const double* partials, int64_t nparts, double* out) {
-    Diag d{0, 0, 0, 0, 0, 1e300, 0, 0};
+    chain_begin();
+    Diag d = diag_none();
     for (int64_t b = threadIdx.x; b < nparts; b += blockDim.x) {
         const double* p = partials + 8 * b;
-        diag_combine(d, Diag{p[0], p[1], p[2], p[3], p[4], p[5], p[6], p[7]});
+        for (int k = 0; k < 5; ++k) d.s[k] += p[k];
+        d.mn = fminf(d.mn, (float)p[5]);  // a float, or 1e300: infinity
+        d.mb = max(d.mb, __double_as_longlong(p[6]));
+        d.bad += (int)p[7];
     }
-    diag_block_reduce(d, out);
+    diag_block_reduce<false>(d, out);
 }
 
 // Block b combines FP32 fluid records [b per, (b + 1) per) and energy
@@ -282,20 +337,29 @@ __global__ void __launch_bounds__(kDiagThreads) diag_finish_kernel(const double*
 __global__ void __launch_bounds__(kDiagThreads) diag_chunk_kernel(const float* rec, int64_t nrec, int64_t per,
                                                                   const float* en, int64_t nen, int64_t per_e,
                                                                   double dxcube, double* scratch) {
-    Diag d{0, 0, 0, 0, 0, 1e300, 0, 0};
+    chain_begin();
+    Diag d = diag_none();
+    float b2 = 0.0f;
     const int64_t b0 = (int64_t)blockIdx.x * per;
     const int64_t b1 = b0 + per < nrec ? b0 + per : nrec;
     for (int64_t b = b0 + threadIdx.x; b < b1; b += blockDim.x) {
         const float4 p = reinterpret_cast<const float4*>(rec)[2 * b];
         const float4 q = reinterpret_cast<const float4*>(rec)[2 * b + 1];
-        diag_combine(d, Diag{p.x, p.y, p.z, p.w, q.x, q.y >= 3.0e38f ? 1e300 : (double)q.y,
-                             sqrt(fmax(0.0, -(double)q.z)), q.w});
+        d.s[0] += p.x;
+        d.s[1] += p.y;
+        d.s[2] += p.z;
+        d.s[3] += p.w;
+        d.s[4] += q.x;
+        if (q.y < 3.0e38f) d.mn = fminf(d.mn, q.y);
+        b2 = fmaxf(b2, -q.z);
+        d.bad += (int)q.w;
     }
+    d.mb = __double_as_longlong((double)b2);
     const int64_t e0 = (int64_t)blockIdx.x * per_e;
     const int64_t e1 = e0 + per_e < nen ? e0 + per_e : nen;
-    for (int64_t b = e0 + threadIdx.x; b < e1; b += blockDim.x) d.en += en[b];
-    d.en *= dxcube;
-    diag_block_reduce(d, scratch + 8 * (int64_t)blockIdx.x);
+    for (int64_t b = e0 + threadIdx.x; b < e1; b += blockDim.x) d.s[4] += en[b];
+    d.s[4] *= dxcube;
+    diag_block_reduce<true>(d, scratch + 8 * (int64_t)blockIdx.x);
 }
 
 // Witness slab: the x range [rows[2 j], rows[2 j + 1]) of each row j in plane
@@ -347,12 +411,10 @@ cudaError_t launch_diag_finish_step(const DiagOut& d, int64_t nrec, cudaStream_t
     if (chunks > kDiagBlocks) chunks = kDiagBlocks;
     const int64_t per = (nrec + chunks - 1) / chunks;
     const int64_t per_e = (d.nenergy + chunks - 1) / chunks;
-    diag_chunk_kernel<<<(unsigned)chunks, kDiagThreads, 0, s>>>(d.records, nrec, per, d.energy, d.nenergy, per_e,
-                                                                d.dxcube, d.scratch);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chained(diag_chunk_kernel, (unsigned)chunks, kDiagThreads, s, (const float*)d.records, nrec, per,
+                                   (const float*)d.energy, d.nenergy, per_e, d.dxcube, d.scratch);
     if (e != cudaSuccess) return e;
-    diag_finish_kernel<<<1, kDiagThreads, 0, s>>>(d.scratch, chunks, d.out);
-    return cudaGetLastError();
+    return launch_chained(diag_finish_kernel, 1, kDiagThreads, s, (const double*)d.scratch, chunks, d.out);
 }
 
 cudaError_t launch_init(const Grid& g, void* f, int storage, float n0, const double* d_profile, int n_profile,
@@ -433,20 +495,26 @@ cudaError_t launch_linecut(const StepArgs& a, int storage, double r, float* out,
     return cudaGetLastError();
 }
 
+template <int ST>
+static cudaError_t diag_t(const StepArgs& a, int blocks, double dxcube, double* partials, cudaStream_t s) {
+    const LinearMap m(a.g);
+    return launch_chained(a.g.periodic ? diag_kernel<ST, true> : diag_kernel<ST, false>, blocks, kDiagThreads, s, a,
+                          m.nxy, m.nx, dxcube, partials);
+}
+
 cudaError_t launch_diag(const StepArgs& a, int storage, double dxcube, double* partials, double* out, cudaStream_t s) {
     const int64_t need = (a.g.N + kDiagThreads - 1) / kDiagThreads;
-    const int blocks = (int)(need < kDiagBlocks ? need : kDiagBlocks);
-    const bool per = a.g.periodic;
+    constexpr int64_t resident = 2 * 152;  // two blocks per SM
+    static_assert(resident <= kDiagBlocks, "partial records");
+    const int blocks = (int)(need < resident ? need : resident);
+    cudaError_t e = cudaErrorInvalidValue;
     switch (storage) {
-        case 0: if (per) diag_kernel<0, true><<<blocks, kDiagThreads, 0, s>>>(a, dxcube, partials); else diag_kernel<0, false><<<blocks, kDiagThreads, 0, s>>>(a, dxcube, partials); break;
-        case 1: if (per) diag_kernel<1, true><<<blocks, kDiagThreads, 0, s>>>(a, dxcube, partials); else diag_kernel<1, false><<<blocks, kDiagThreads, 0, s>>>(a, dxcube, partials); break;
-        case 2: if (per) diag_kernel<2, true><<<blocks, kDiagThreads, 0, s>>>(a, dxcube, partials); else diag_kernel<2, false><<<blocks, kDiagThreads, 0, s>>>(a, dxcube, partials); break;
-        default: return cudaErrorInvalidValue;
+        case 0: e = diag_t<0>(a, blocks, dxcube, partials, s); break;
+        case 1: e = diag_t<1>(a, blocks, dxcube, partials, s); break;
+        case 2: e = diag_t<2>(a, blocks, dxcube, partials, s); break;
     }
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    diag_finish_kernel<<<1, kDiagThreads, 0, s>>>(partials, blocks, out);
-    return cudaGetLastError();
+    return launch_chained(diag_finish_kernel, 1, kDiagThreads, s, (const double*)partials, (int64_t)blocks, out);
 }
 
 }  // namespace pwfa

@@ -79,16 +79,9 @@ __global__ void __launch_bounds__(kLinearThreads, FluidOcc<ST, COLL>::blocks)
     float v[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 3.0e38f, 3.0e38f, 0.0f};
     if (m.node(a.g, x, y, z)) {
         NodeDiag nd;
+        nd.fields = fields != 0;
         fluid_node<ST, COLL, PER, true>(a, x, y, z, &nd);
-        if (fields) {
-            const int64_t o = ((int64_t)z * a.g.ny + y) * a.g.nx + x;
-            float e2 = 0.0f;
-            for (int c = 0; c < 3; ++c) {
-                const float ev = __ldg(a.E[c] + o), bv = __ldg(a.Bc[c] + o);
-                e2 += ev * ev + bv * bv;
-            }
-            v[4] = 0.5f * e2;
-        }
+        v[4] = 0.5f * nd.e2;
         const bool fin = isfinite(nd.n) && isfinite(nd.a1) && isfinite(nd.a2) && isfinite(nd.a3);
         v[0] = nd.n; v[1] = nd.a1; v[2] = nd.a2; v[3] = nd.a3;
         v[5] = nd.n;

@@ -22,6 +22,8 @@ static_assert(kLinearThreads <= PWFA_FLUID_MAX_THREADS, "launch bounds");
 // Node quantities handed to the fused diagnostics (state entering the step).
 struct NodeDiag {
     float n, a1, a2, a3, beta2;
+    bool fields;  // in: the field energy is wanted
+    float e2;     // |E|^2 + |Bc|^2 of the components stored at the node
 };
 
 // m = sum_i xi_i f_i over one lattice's 19 values (signed adds, q ascending).
@@ -148,6 +150,18 @@ __device__ __forceinline__ void fluid_rest(const StepArgs& a, int x, int y, int 
         F[0] = -n * (e[0] + beta[1] * b2 - beta[2] * b1);
         F[1] = -n * (e[1] + beta[2] * b0 - beta[0] * b2);
         F[2] = -n * (e[2] + beta[0] * b1 - beta[1] * b0);
+    }
+    if (DIAG) {
+        // beside the node averages, which have just read these values (at the
+        // end of the node they were a memory round of their own)
+        nd->e2 = 0.0f;
+        if (nd->fields) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float ev = __ldg(a.E[c] + node), bv = __ldg(a.Bc[c] + node);
+                nd->e2 += ev * ev + bv * bv;
+            }
+        }
     }
 
     const int64_t LS = lattice_stride(g);
