@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kBatchTile, PHASE == 1 ? BatchFluidOcc<ST, COL
         int x, y, z;
         if (!tile_node(sa.g, t, tid, x, y, z)) continue;
         if (PHASE == 0) faraday_node<PER>(sa, x, y, z);
-        else if (PHASE == 1) fluid_node<ST, COLL, PER, false, false, BatchFluidOcc<ST, COLL>::park>(sa, x, y, z);
+        else if (PHASE == 1) fluid_node<ST, COLL, PER, false, false, BatchFluidOcc<ST, COLL>::park, true>(sa, x, y, z);
         else ampere_node<PER>(sa, x, y, z, s_zc);
     }
 }

@@ -90,6 +90,17 @@ __device__ __forceinline__ void fluid_moments(const StepArgs& a, const float (&f
 // Shared-memory words of one thread's parked BGK values (lattices 2 and 3).
 constexpr int kStashVals = 2 * kQ;
 
+// FP32 results of a step. Plain stores in the kernels of one instance,
+// streaming ones (CS) in the batch, where the next phase starts far from what
+// this one wrote last: fluid kernel on GB300, streaming / plain, 512x256x256
+// regularized 3176 / 3138 us, 256x128x128 BGK 408 / 406, 203x97x131 254.8 /
+// 253.6; 32 batched instances 5358 / 5417.
+template <bool CS>
+__device__ __forceinline__ void put(float* p, float v) {
+    if (CS) __stcs(p, v);
+    else *p = v;
+}
+
 // Everything after the moments: source, collision, stores, current. f holds
 // the pulled populations f^n(x) (of the clamped node when bnd; BGK and
 // stream-only read them, the regularized form only uses f as its output
@@ -97,7 +108,8 @@ constexpr int kStashVals = 2 * kQ;
 // and the post-collision values are formed in stored units too, so that
 // neither the decode nor the encode of the deviations costs a per-value
 // operation.
-template <int ST, int COLL, bool PER, bool DIAG = false, bool RAW = false, bool MOM = false, bool PARK = false>
+template <int ST, int COLL, bool PER, bool DIAG = false, bool RAW = false, bool MOM = false, bool PARK = false,
+          bool CS = false>
 __device__ __forceinline__ void fluid_rest(const StepArgs& a, int x, int y, int z, float (&f)[kL][kQ], bool bnd,
                                            NodeMoments& s, NodeDiag* nd = nullptr) {
     using T = typename Codec<ST>::T;
@@ -126,7 +138,7 @@ __device__ __forceinline__ void fluid_rest(const StepArgs& a, int x, int y, int 
         // the adjoint's recompute keeps the lattice sums (the reverse step
         // needs nothing else of the populations)
 #pragma unroll
-        for (int l = 0; l < kL; ++l) __stcs(a.mom + (int64_t)l * g.N + node, A[l]);
+        for (int l = 0; l < kL; ++l) a.mom[(int64_t)l * g.N + node] = A[l];
     }
     if (DIAG) {
         nd->n = A[0];
@@ -258,7 +270,7 @@ __device__ __forceinline__ void fluid_rest(const StepArgs& a, int x, int y, int 
             // (stream only: f* = f)
             if constexpr (ST == 0) {
 #pragma unroll
-                for (int q = 0; q < kQ; ++q) Codec<ST>::store(fo[l] + pop_off(q, node), f[l][q], l, q, a.n0);
+                for (int q = 0; q < kQ; ++q) put<CS>(fo[l] + pop_off(q, node), f[l][q]);
             }
         }
         if constexpr (RAWR) {
@@ -277,21 +289,22 @@ __device__ __forceinline__ void fluid_rest(const StepArgs& a, int x, int y, int 
     const float ps1 = (A[2] + F[1] * a.dt) * inn;
     const float ps2 = (A[3] + F[2] * a.dt) * inn;
     const float ngs = -n * rsqrtf(1.0f + ps0 * ps0 + ps1 * ps1 + ps2 * ps2);
-    __stcs(a.J[0] + node, ngs * ps0);
-    __stcs(a.J[1] + node, ngs * ps1);
-    __stcs(a.J[2] + node, ngs * ps2);
+    put<CS>(a.J[0] + node, ngs * ps0);
+    put<CS>(a.J[1] + node, ngs * ps1);
+    put<CS>(a.J[2] + node, ngs * ps2);
 }
 
 // Everything after the gather: moments, then fluid_rest.
-template <int ST, int COLL, bool PER, bool DIAG = false, bool RAW = false, bool MOM = false, bool PARK = false>
+template <int ST, int COLL, bool PER, bool DIAG = false, bool RAW = false, bool MOM = false, bool PARK = false,
+          bool CS = false>
 __device__ __forceinline__ void fluid_compute(const StepArgs& a, int x, int y, int z, float (&f)[kL][kQ], bool bnd,
                                               NodeDiag* nd = nullptr) {
     NodeMoments s;
     fluid_moments<ST, COLL, RAW>(a, f, s);
-    fluid_rest<ST, COLL, PER, DIAG, RAW, MOM, PARK>(a, x, y, z, f, bnd, s, nd);
+    fluid_rest<ST, COLL, PER, DIAG, RAW, MOM, PARK, CS>(a, x, y, z, f, bnd, s, nd);
 }
 
-template <int ST, int COLL, bool PER, bool DIAG = false, bool MOM = false, bool PARK = false>
+template <int ST, int COLL, bool PER, bool DIAG = false, bool MOM = false, bool PARK = false, bool CS = false>
 __device__ __forceinline__ void fluid_node(const StepArgs& a, int x, int y, int z, NodeDiag* nd = nullptr) {
     using T = typename Codec<ST>::T;
     float f[kL][kQ];
@@ -299,7 +312,7 @@ __device__ __forceinline__ void fluid_node(const StepArgs& a, int x, int y, int 
     // the 16-bit regularized form works in stored units (see fluid_compute)
     constexpr bool RAW = ST != 0 && COLL == 1;
     gather<ST, PER, RAW>(a.g, static_cast<const T*>(a.fin), a.n0, x, y, z, f, bnd, a.src_shift, a.dbg);
-    fluid_compute<ST, COLL, PER, DIAG, RAW, MOM, PARK>(a, x, y, z, f, bnd, nd);
+    fluid_compute<ST, COLL, PER, DIAG, RAW, MOM, PARK, CS>(a, x, y, z, f, bnd, nd);
 }
 
 }  // namespace pwfa

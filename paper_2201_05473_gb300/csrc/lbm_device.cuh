@@ -53,7 +53,7 @@ template <int ST> struct Codec;
 template <> struct Codec<0> {
     using T = float;
     static __device__ __forceinline__ float load(const T* p, int, int, float) { return __ldg(p); }
-    static __device__ __forceinline__ void store(T* p, float v, int, int, float) { __stcs(p, v); }
+    static __device__ __forceinline__ void store(T* p, float v, int, int, float) { *p = v; }
 };
 // The 16-bit codecs also move the pair of lattices (l0, l0 + 1) that share a
 // 32-bit word (see pop_elem): p points at the word's first (even) element.
