@@ -62,7 +62,8 @@ KERNEL_SOURCES = ["paper_2201_05473_gb300/csrc/fluid.cu", "paper_2201_05473_gb30
                   "paper_2201_05473_gb300/csrc/lbm_node.cuh", "paper_2201_05473_gb300/csrc/lbm_device.cuh"]
 # the fused field kernel (Ampere with the next step's Faraday): 60 B/node
 FIELD_TRAFFIC_FILE = os.path.join(ROOT, "profiles", "ampere_faraday_kernel_traffic.json")
-FIELD_SOURCES = ["paper_2201_05473_gb300/csrc/fields.cu", "paper_2201_05473_gb300/csrc/fields_fused.cuh",
+FIELD_SOURCES = ["paper_2201_05473_gb300/csrc/fields.cu", "paper_2201_05473_gb300/csrc/fields_rows.cuh",
+                 "paper_2201_05473_gb300/csrc/fields_fused.cuh",
                  "paper_2201_05473_gb300/csrc/fields_node.cuh", "paper_2201_05473_gb300/csrc/lbm_device.cuh"]
 FIELD_BYTES = 60
 
