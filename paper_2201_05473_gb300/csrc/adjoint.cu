@@ -402,12 +402,12 @@ __global__ void __launch_bounds__(kLinearThreads, 4) adj_fluid_kernel(const AdjA
             }
             const uint32_t off = pop_off(q, PWFA_CHECK(s.dbg, src, 0, g.Np, 7u));
 #pragma unroll
-            for (int l = 0; l < kL; ++l) S[l][q] = __ldg(a.Fbar_in + l * LS + off);
+            for (int l = 0; l < kL; ++l) S[l][q] = ld_state(a.Fbar_in + l * LS + off);
         }
         // the lattice sums of the node's pulled populations, as the forward
         // step formed them (for a boundary node: of its clamped node's)
 #pragma unroll
-        for (int l = 0; l < kL; ++l) A[l] = __ldg(s.mom + (int64_t)l * g.N + node);
+        for (int l = 0; l < kL; ++l) A[l] = ld_state(s.mom + (int64_t)l * g.N + node);
     } else {
 #pragma unroll
         for (int l = 0; l < kL; ++l)
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kLinearThreads, 4) adj_fluid_kernel(const AdjA
     const bool forced = (COLL != 2) && s.couple;
     if (act) {
         float e[3] = {0.0f, 0.0f, 0.0f}, b[3] = {0.0f, 0.0f, 0.0f}, F[3] = {0.0f, 0.0f, 0.0f};
-        const float Jb[3] = {__ldg(a.Jbar[0] + node), __ldg(a.Jbar[1] + node), __ldg(a.Jbar[2] + node)};
+        const float Jb[3] = {ld_state(a.Jbar[0] + node), ld_state(a.Jbar[1] + node), ld_state(a.Jbar[2] + node)};
         if (forced) {
             float bc[3], bn[3];
             node_E<PER>(g, s.E, x, y, z, e, s.dbg);
@@ -729,23 +729,23 @@ __device__ __forceinline__ void adj_fe_load(const AdjArgs& a, int o, int pi, int
     pk = (int)PWFA_CHECK(a.f.dbg, o + pi + pj + pk, 0, a.f.g.N, 7u) - o - pi - pj;
 #endif
     const float *bx = a.bbar[0], *by = a.bbar[1], *bz = a.bbar[2];
-    v.x2 = __ldg(bx + o + pk);
-    v.x3 = __ldg(bx + o + pj + pk);
-    v.y2 = __ldg(by + o + pk);
-    v.y3 = __ldg(by + o + pi + pk);
-    v.z0 = __ldg(bz + o);
-    v.z1 = __ldg(bz + o + pi);
-    v.z2 = __ldg(bz + o + pj);
-    v.z3 = __ldg(bz + o + pi + pj);
-    v.bn0 = __ldg(a.Bnp[0] + o);
-    v.bn1 = __ldg(a.Bnp[1] + o);
-    v.bn2 = __ldg(a.Bnp[2] + o);
-    v.ez1 = own ? __ldg(a.ebar[2] + o + pk) : 0.0f;
+    v.x2 = ld_state(bx + o + pk);
+    v.x3 = ld_state(bx + o + pj + pk);
+    v.y2 = ld_state(by + o + pk);
+    v.y3 = ld_state(by + o + pi + pk);
+    v.z0 = ld_state(bz + o);
+    v.z1 = ld_state(bz + o + pi);
+    v.z2 = ld_state(bz + o + pj);
+    v.z3 = ld_state(bz + o + pi + pj);
+    v.bn0 = ld_state(a.Bnp[0] + o);
+    v.bn1 = ld_state(a.Bnp[1] + o);
+    v.bn2 = ld_state(a.Bnp[2] + o);
+    v.ez1 = own ? ld_state(a.ebar[2] + o + pk) : 0.0f;
     if (slab) {
-        v.ex0 = __ldg(a.ebar[0] + o);
-        v.ex1 = __ldg(a.ebar[0] + o + pi);
-        v.ey0 = __ldg(a.ebar[1] + o);
-        v.ey1 = __ldg(a.ebar[1] + o + pj);
+        v.ex0 = ld_state(a.ebar[0] + o);
+        v.ex1 = ld_state(a.ebar[0] + o + pi);
+        v.ey0 = ld_state(a.ebar[1] + o);
+        v.ey1 = ld_state(a.ebar[1] + o + pj);
         v.E0 = a.Ebar[0][o];
         v.E1 = a.Ebar[1][o];
         v.E2 = a.Ebar[2][o];
@@ -790,11 +790,11 @@ __global__ void __launch_bounds__(kRX * kRY, PWFA_ADJ_FE_MIN_BLOCKS) adj_faces_e
 #ifdef PWFA_DEBUG
         oc = (int)PWFA_CHECK(a.f.dbg, oc + pi + pj, 0, g.N, 7u) - pi - pj;
 #endif
-        x0 = __ldg(a.bbar[0] + oc);
-        x1 = __ldg(a.bbar[0] + oc + pj);
-        y0 = __ldg(a.bbar[1] + oc);
-        y1 = __ldg(a.bbar[1] + oc + pi);
-        ez0 = own && kfirst >= kz0 ? __ldg(a.ebar[2] + oc) : 0.0f;
+        x0 = ld_state(a.bbar[0] + oc);
+        x1 = ld_state(a.bbar[0] + oc + pj);
+        y0 = ld_state(a.bbar[1] + oc);
+        y1 = ld_state(a.bbar[1] + oc + pi);
+        ez0 = own && kfirst >= kz0 ? ld_state(a.ebar[2] + oc) : 0.0f;
     }
     AdjFEPlane nxt;
     adj_fe_load(a, o, pi, pj, pk, own, own && kfirst >= kz0, nxt);

@@ -113,8 +113,8 @@ __global__ void __launch_bounds__(kLinearThreads) import_f_kernel(Grid g, const 
 #pragma unroll
     for (int q = 0; q < kQ; ++q) {
         const int64_t o = q * g.N + ox[xi_x(q) + 1] + oy[xi_y(q) + 1] + oz[xi_z(q) + 1];
-        v0[q] = __ldg(p0 + o);
-        v1[q] = __ldg(p1 + o);
+        v0[q] = ld_state(p0 + o);
+        v1[q] = ld_state(p1 + o);
     }
     const int64_t LS = lattice_stride(g);
 #pragma unroll
@@ -293,8 +293,8 @@ __global__ void __launch_bounds__(kDiagThreads, 2)
             float e[6];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                e[c] = __ldg(a.E[c] + node);
-                e[3 + c] = __ldg(a.Bc[c] + node);
+                e[c] = ld_state(a.E[c] + node);
+                e[3 + c] = ld_state(a.Bc[c] + node);
             }
             float A[kL], inn;
             node_moments(f, a.n_floor, A, inn, beta);

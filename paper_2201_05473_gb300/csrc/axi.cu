@@ -52,22 +52,22 @@ __device__ __forceinline__ void load_fields(const Args& a, int k, int j, NodeFie
     const int64_t o = (int64_t)k * nr + j;
     const int64_t km = k > 0 ? -nr : 0, kp = k < a.nz - 1 ? nr : 0;
     const int jm = j > 0 ? -1 : 0, jp = j < nr - 1 ? 1 : 0;
-    v.er[0][0] = __ldg(a.Er + o + km + jm);
-    v.er[0][1] = __ldg(a.Er + o + km);
-    v.er[1][0] = __ldg(a.Er + o + jm);
-    v.er[1][1] = __ldg(a.Er + o);
-    v.er[2][0] = __ldg(a.Er + o + kp + jm);
-    v.er[2][1] = __ldg(a.Er + o + kp);
-    v.ez[0][0] = __ldg(a.Ez + o + km + jm);
-    v.ez[0][1] = __ldg(a.Ez + o + km);
-    v.ez[0][2] = __ldg(a.Ez + o + km + jp);
-    v.ez[1][0] = __ldg(a.Ez + o + jm);
-    v.ez[1][1] = __ldg(a.Ez + o);
-    v.ez[1][2] = __ldg(a.Ez + o + jp);
-    v.bt[0][0] = __ldg(a.Bt + o + km + jm);
-    v.bt[0][1] = __ldg(a.Bt + o + km);
-    v.bt[1][0] = __ldg(a.Bt + o + jm);
-    v.bt[1][1] = __ldg(a.Bt + o);
+    v.er[0][0] = ld_state(a.Er + o + km + jm);
+    v.er[0][1] = ld_state(a.Er + o + km);
+    v.er[1][0] = ld_state(a.Er + o + jm);
+    v.er[1][1] = ld_state(a.Er + o);
+    v.er[2][0] = ld_state(a.Er + o + kp + jm);
+    v.er[2][1] = ld_state(a.Er + o + kp);
+    v.ez[0][0] = ld_state(a.Ez + o + km + jm);
+    v.ez[0][1] = ld_state(a.Ez + o + km);
+    v.ez[0][2] = ld_state(a.Ez + o + km + jp);
+    v.ez[1][0] = ld_state(a.Ez + o + jm);
+    v.ez[1][1] = ld_state(a.Ez + o);
+    v.ez[1][2] = ld_state(a.Ez + o + jp);
+    v.bt[0][0] = ld_state(a.Bt + o + km + jm);
+    v.bt[0][1] = ld_state(a.Bt + o + km);
+    v.bt[1][0] = ld_state(a.Bt + o + jm);
+    v.bt[1][1] = ld_state(a.Bt + o);
 }
 
 // Faraday on the face (k - 1 + K, j - 1 + J): B_theta(t_{n+1}) = B_theta(t_n) +
@@ -86,7 +86,7 @@ __device__ __forceinline__ void pull(const Args& a, int64_t c, float (&f)[kL][kQ
     for (int q = 0; q < kQ; ++q) {
         const float* p = a.fin + chunk(c - xz(q) * a.nr - xr(q));
 #pragma unroll
-        for (int l = 0; l < kL; ++l) f[l][q] = __ldg(p + (l * kQ + q) * kPopStride);
+        for (int l = 0; l < kL; ++l) f[l][q] = ld_state(p + (l * kQ + q) * kPopStride);
     }
 }
 
@@ -283,16 +283,16 @@ __global__ void __launch_bounds__(kAmpThreads) ampere_kernel(const Args a) {
     if (k0 >= a.nz || j < 1 || j > a.nr - 2) return;  // (the walls keep their zeros)
     const int64_t o = (int64_t)k0 * a.nr + j;
     float bt[kAmpRows + 1], bt_j[kAmpRows], jr[kAmpRows], jr_j[kAmpRows], jz[kAmpRows + 1], er[kAmpRows], ez[kAmpRows];
-    bt[0] = __ldg(a.Btn + o - (k0 > 0 ? a.nr : 0));
-    jz[kAmpRows] = __ldg(a.Jz + (int64_t)min(k0 + kAmpRows, a.nz - 1) * a.nr + j);
+    bt[0] = ld_state(a.Btn + o - (k0 > 0 ? a.nr : 0));
+    jz[kAmpRows] = ld_state(a.Jz + (int64_t)min(k0 + kAmpRows, a.nz - 1) * a.nr + j);
 #pragma unroll
     for (int i = 0; i < kAmpRows; ++i) {
         const int64_t p = (int64_t)min(k0 + i, a.nz - 1) * a.nr + j;
-        bt[i + 1] = __ldg(a.Btn + p);
-        bt_j[i] = __ldg(a.Btn + p - 1);
-        jr[i] = __ldg(a.Jr + p);
-        jr_j[i] = __ldg(a.Jr + p + 1);
-        jz[i] = __ldg(a.Jz + p);
+        bt[i + 1] = ld_state(a.Btn + p);
+        bt_j[i] = ld_state(a.Btn + p - 1);
+        jr[i] = ld_state(a.Jr + p);
+        jr_j[i] = ld_state(a.Jr + p + 1);
+        jz[i] = ld_state(a.Jz + p);
         er[i] = a.ErO[p];
         ez[i] = a.EzO[p];
     }

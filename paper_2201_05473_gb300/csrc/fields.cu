@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kBX * kBY) faraday_energy_kernel(const StepArg
         faraday_node<PER>(a, i, j, blockIdx.z);
         const int64_t o = ((int64_t)blockIdx.z * a.g.ny + j) * a.g.nx + i;
         for (int c = 0; c < 3; ++c) {
-            const float ev = __ldg(a.E[c] + o), bv = __ldg(a.Bc[c] + o);
+            const float ev = ld_state(a.E[c] + o), bv = ld_state(a.Bc[c] + o);
             e2 += ev * ev + bv * bv;
         }
         e2 *= 0.5f;

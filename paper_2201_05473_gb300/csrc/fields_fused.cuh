@@ -61,21 +61,21 @@ __device__ __forceinline__ void af_load(const StepArgs& a, int o, int zp, int xm
     yp = PWFA_CHECK(a.dbg, o + yp, 0, a.g.N, 6u) - o;
     zp = PWFA_CHECK(a.dbg, o + zp, 0, a.g.N, 6u) - o;
 #endif
-    v.e0 = __ldg(a.E[0] + o);
-    v.e1 = __ldg(a.E[1] + o);
-    v.e2 = __ldg(a.E[2] + o);
-    v.bx = __ldg(Bx + o);
-    v.by = __ldg(By + o);
-    v.bz = __ldg(Bz + o);
-    v.bz_i = __ldg(Bz + o + xm);
-    v.by_i = __ldg(By + o + xm);
-    v.bz_j = __ldg(Bz + o + ym);
-    v.bx_j = __ldg(Bx + o + ym);
-    v.j0 = __ldg(a.J[0] + o);
-    v.j0_i = __ldg(a.J[0] + o + xp);
-    v.j1 = __ldg(a.J[1] + o);
-    v.j1_j = __ldg(a.J[1] + o + yp);
-    v.j2k = __ldg(a.J[2] + o + zp);
+    v.e0 = ld_state(a.E[0] + o);
+    v.e1 = ld_state(a.E[1] + o);
+    v.e2 = ld_state(a.E[2] + o);
+    v.bx = ld_state(Bx + o);
+    v.by = ld_state(By + o);
+    v.bz = ld_state(Bz + o);
+    v.bz_i = ld_state(Bz + o + xm);
+    v.by_i = ld_state(By + o + xm);
+    v.bz_j = ld_state(Bz + o + ym);
+    v.bx_j = ld_state(Bx + o + ym);
+    v.j0 = ld_state(a.J[0] + o);
+    v.j0_i = ld_state(a.J[0] + o + xp);
+    v.j1 = ld_state(a.J[1] + o);
+    v.j1_j = ld_state(a.J[1] + o + yp);
+    v.j2k = ld_state(a.J[2] + o + zp);
 }
 
 // The fused step over one tile (tile coordinates tbx, tby, tbz): called by
@@ -130,9 +130,9 @@ __device__ __forceinline__ void ampere_faraday_tile(const StepArgs& a, const Fie
 #ifdef PWFA_DEBUG
         zm = PWFA_CHECK(a.dbg, o + zm, -guard_elems(g), g.N, 6u) - o;
 #endif
-        bp0 = __ldg(a.Bn[0] + o + zm);
-        bp1 = __ldg(a.Bn[1] + o + zm);
-        j2n = __ldg(a.J[2] + o);
+        bp0 = ld_state(a.Bn[0] + o + zm);
+        bp1 = ld_state(a.Bn[1] + o + zm);
+        j2n = ld_state(a.J[2] + o);
     }
     // the loads of the first plane; each iteration issues the next plane's
     // before it works on its own

@@ -17,7 +17,7 @@ namespace pwfa {
 template <bool PER>
 __device__ __forceinline__ float yee_ld(const Grid& g, const float* a, int i, int j, int k) {
     if (PER) { i = wrapi(i, g.nx); j = wrapi(j, g.ny); k = wrapi(k, g.nz); }
-    return __ldg(a + ((int64_t)k * g.ny + j) * g.nx + i);
+    return ld_state(a + ((int64_t)k * g.ny + j) * g.nx + i);
 }
 
 // Neighbour indices: wrapped by yee_ld on periodic grids, clamped into the
@@ -101,11 +101,11 @@ __device__ __forceinline__ void faraday_node(const StepArgs& a, int i, int j, in
     pj = PWFA_CHECK(a.dbg, o + pj, 0, g.N, 4u) - o;
     pk = PWFA_CHECK(a.dbg, o + pk, 0, g.N, 4u) - o;
 #endif
-    const float ex = __ldg(Ex + o), ey = __ldg(Ey + o), ez = __ldg(Ez + o);
-    const float ez_j = __ldg(Ez + o + pj), ey_k = __ldg(Ey + o + pk);
-    const float ex_k = __ldg(Ex + o + pk), ez_i = __ldg(Ez + o + pi);
-    const float ey_i = __ldg(Ey + o + pi), ex_j = __ldg(Ex + o + pj);
-    const float b[3] = {__ldg(a.Bc[0] + o), __ldg(a.Bc[1] + o), __ldg(a.Bc[2] + o)};
+    const float ex = ld_state(Ex + o), ey = ld_state(Ey + o), ez = ld_state(Ez + o);
+    const float ez_j = ld_state(Ez + o + pj), ey_k = ld_state(Ey + o + pk);
+    const float ex_k = ld_state(Ex + o + pk), ez_i = ld_state(Ez + o + pi);
+    const float ey_i = ld_state(Ey + o + pi), ex_j = ld_state(Ex + o + pj);
+    const float b[3] = {ld_state(a.Bc[0] + o), ld_state(a.Bc[1] + o), ld_state(a.Bc[2] + o)};
     float bn[3];
     faraday_values<PER>(g, a.cdt, i, j, k, b, ex, ey, ez, ez_j, ey_k, ex_k, ez_i, ey_i, ex_j, bn);
     a.Bn[0][o] = bn[0];
@@ -152,22 +152,22 @@ __device__ __forceinline__ AmpereIn ampere_loads(const StepArgs& a, int i, int j
         uk = PWFA_CHECK(a.dbg, o + uk, 0, g.N, 5u) - o;
         (void)di; (void)dj; (void)ui; (void)uj;
 #endif
-        v.bz_j = __ldg(Bz + o - dj);
-        v.by_k = __ldg(By + o - dk);
-        v.bx_k = __ldg(Bx + o - dk);
-        v.bz_i = __ldg(Bz + o - di);
-        v.by_i = __ldg(By + o - di);
-        v.bx_j = __ldg(Bx + o - dj);
-        v.j0_i = __ldg(a.J[0] + o + ui);
-        v.j1_j = __ldg(a.J[1] + o + uj);
-        v.j2_k = __ldg(a.J[2] + o + uk);
+        v.bz_j = ld_state(Bz + o - dj);
+        v.by_k = ld_state(By + o - dk);
+        v.bx_k = ld_state(Bx + o - dk);
+        v.bz_i = ld_state(Bz + o - di);
+        v.by_i = ld_state(By + o - di);
+        v.bx_j = ld_state(Bx + o - dj);
+        v.j0_i = ld_state(a.J[0] + o + ui);
+        v.j1_j = ld_state(a.J[1] + o + uj);
+        v.j2_k = ld_state(a.J[2] + o + uk);
     }
-    v.bx = __ldg(Bx + o);
-    v.by = __ldg(By + o);
-    v.bz = __ldg(Bz + o);
-    v.j0 = __ldg(a.J[0] + o);
-    v.j1 = __ldg(a.J[1] + o);
-    v.j2 = __ldg(a.J[2] + o);
+    v.bx = ld_state(Bx + o);
+    v.by = ld_state(By + o);
+    v.bz = ld_state(Bz + o);
+    v.j0 = ld_state(a.J[0] + o);
+    v.j1 = ld_state(a.J[1] + o);
+    v.j2 = ld_state(a.J[2] + o);
     v.e0 = a.E[0][o];
     v.e1 = a.E[1][o];
     v.e2 = a.E[2][o];

@@ -28,13 +28,13 @@ constexpr int kARLanes = 31;
 template <int V>
 __device__ __forceinline__ void row_ld(float (&d)[V], const float* p) {
     if constexpr (V == 4) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+        const float4 t = ld_state(reinterpret_cast<const float4*>(p));
         d[0] = t.x; d[1] = t.y; d[2] = t.z; d[3] = t.w;
     } else if constexpr (V == 2) {
-        const float2 t = __ldg(reinterpret_cast<const float2*>(p));
+        const float2 t = ld_state(reinterpret_cast<const float2*>(p));
         d[0] = t.x; d[1] = t.y;
     } else {
-        d[0] = __ldg(p);
+        d[0] = ld_state(p);
     }
 }
 template <int V>
@@ -103,8 +103,8 @@ __device__ __forceinline__ void ar_load(const StepArgs& a, int o, int xp, int yp
     row_ld(v.j0, a.J[0] + o);
     row_ld(v.j1, a.J[1] + o);
     row_ld(v.j1_j, a.J[1] + o + yp);
-    v.bz_f = first ? __ldg(Bz + o - 1) : 0.0f;
-    if (V == 1) v.j0_l = __ldg(a.J[0] + o + xp);
+    v.bz_f = first ? ld_state(Bz + o - 1) : 0.0f;
+    if (V == 1) v.j0_l = ld_state(a.J[0] + o + xp);
     if (HALO) {
         row_ld(v.e2, a.E[2] + o);
         row_ld(v.bx_j, Bx + o - nx);
@@ -116,9 +116,9 @@ __device__ __forceinline__ void ar_load(const StepArgs& a, int o, int xp, int yp
         row_ld(v.ybz, Bz + o + yp);
         row_ld(v.yj0, a.J[0] + o + yp);
         row_ld(v.yj2_k, a.J[2] + o + yp + zp);
-        v.by_f = first ? __ldg(By + o - 1) : 0.0f;
-        v.yby_f = first ? __ldg(By + o + yp - 1) : 0.0f;
-        if (V == 1) v.yj0_l = __ldg(a.J[0] + o + yp + xp);
+        v.by_f = first ? ld_state(By + o - 1) : 0.0f;
+        v.yby_f = first ? ld_state(By + o + yp - 1) : 0.0f;
+        if (V == 1) v.yj0_l = ld_state(a.J[0] + o + yp + xp);
     }
 }
 

@@ -170,7 +170,7 @@ __device__ __forceinline__ void fluid_rest(const StepArgs& a, int x, int y, int 
         if (nd->fields) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const float ev = __ldg(a.E[c] + node), bv = __ldg(a.Bc[c] + node);
+                const float ev = ld_state(a.E[c] + node), bv = ld_state(a.Bc[c] + node);
                 nd->e2 += ev * ev + bv * bv;
             }
         }

@@ -7,6 +7,15 @@
 // its writes are visible: the same order as a plain launch, without the
 // launch latency and the ramp between the two. Behind a kernel that is not
 // chained, a copy or an event the launch is ordered as usual.
+//
+// What makes that order sound: griddepcontrol.wait holds a thread until the
+// prerequisite grids have completed and their memory operations are performed
+// and visible to its grid (PTX ISA, griddepcontrol); every thread of every
+// chained kernel waits first thing, so the order carries over from kernel to
+// kernel; the compiler keeps later accesses behind the wait (volatile, with a
+// memory clobber); and what a predecessor may have written is read with
+// coherent loads (ld_state or plain ones), not through the read-only path,
+// whose data must not change while the kernel runs.
 #pragma once
 
 #include <utility>

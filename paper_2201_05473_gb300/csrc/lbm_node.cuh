@@ -52,7 +52,7 @@ __device__ __forceinline__ int64_t src_index(const Grid& g, int x, int y, int z,
 // RAW (16-bit storage): the values are left in stored units (the
 // deviation, scaled for FP16) for a caller that works in those units.
 template <int ST, bool PER, bool RAW = false>
-__device__ __forceinline__ void gather(const Grid& g, const typename Codec<ST>::T* __restrict__ fin,
+__device__ __forceinline__ void gather(const Grid& g, const typename Codec<ST>::T* fin,
                                        float n0, int x, int y, int z, float f[kL][kQ], bool& bnd,
                                        uint32_t src_shift = 0, unsigned* dbg = nullptr) {
     using T = typename Codec<ST>::T;
@@ -66,8 +66,8 @@ __device__ __forceinline__ void gather(const Grid& g, const typename Codec<ST>::
     }
     const int64_t LS = lattice_stride(g);
     // per-lattice (FP32) or per-pair (16-bit) base pointers; 32-bit offsets
-    const T* __restrict__ fl[kL] = {fin, fin + LS, fin + 2 * LS, fin + 3 * LS};
-    const T* __restrict__ fp[2] = {fin, fin + 2 * LS};
+    const T* fl[kL] = {fin, fin + LS, fin + 2 * LS, fin + 3 * LS};
+    const T* fp[2] = {fin, fin + 2 * LS};
     const uint32_t sxy = (uint32_t)g.nx * (uint32_t)g.ny;
     const uint32_t nodec =
         ((uint32_t)zs * (uint32_t)g.ny + (uint32_t)ys) * (uint32_t)g.nx + (uint32_t)xs + (PER ? 0u : src_shift);
@@ -144,13 +144,16 @@ __device__ __forceinline__ float yat(const Grid& g, const float* a, int i, int j
     } else if (i < 0 || j < 0 || k < 0) {
         return 0.0f;
     }
-    return __ldg(a + ((int64_t)k * g.ny + j) * g.nx + i);
+    return ld_state(a + ((int64_t)k * g.ny + j) * g.nx + i);
 }
 
 // Open grids keep a zero guard in front of every Yee array (one plane, one
 // row and one element) and every component outside the conducting box at
 // zero, so the indices just below the grid (x-1, y-1, z-1 and their
 // combinations, wrapping into the previous row/plane or the guard) read 0.
+// Plain loads, coherent as ld_state's but the compiler's to place: opaque ones
+// here cost the BGK form 2 to 4 % (203x97x131 FP32 289.2 -> 297.2 us per step,
+// 256x128x128 BF16 310 -> 323).
 template <bool PER>
 __device__ __forceinline__ void node_E(const Grid& g, const float* const E[3], int x, int y, int z, float e[3],
                                        unsigned* dbg = nullptr) {
@@ -164,9 +167,9 @@ __device__ __forceinline__ void node_E(const Grid& g, const float* const E[3], i
 #ifdef PWFA_DEBUG
         PWFA_CHECK(dbg, o - sxy, -guard_elems(g), g.N, 3u);
 #endif
-        e[0] = 0.5f * (__ldg(E[0] + o - 1) + __ldg(E[0] + o));
-        e[1] = 0.5f * (__ldg(E[1] + o - g.nx) + __ldg(E[1] + o));
-        e[2] = 0.5f * (__ldg(E[2] + o - sxy) + __ldg(E[2] + o));
+        e[0] = 0.5f * (E[0][o - 1] + E[0][o]);
+        e[1] = 0.5f * (E[1][o - g.nx] + E[1][o]);
+        e[2] = 0.5f * (E[2][o - sxy] + E[2][o]);
     }
 }
 
@@ -191,9 +194,9 @@ __device__ __forceinline__ void node_B_sum(const Grid& g, const float* const B[3
         const float* b0 = B[0] + o;
         const float* b1 = B[1] + o;
         const float* b2 = B[2] + o;
-        b[0] = __ldg(b0) + __ldg(b0 - sx) + __ldg(b0 - sxy) + __ldg(b0 - sx - sxy);
-        b[1] = __ldg(b1) + __ldg(b1 - 1) + __ldg(b1 - sxy) + __ldg(b1 - 1 - sxy);
-        b[2] = __ldg(b2) + __ldg(b2 - 1) + __ldg(b2 - sx) + __ldg(b2 - 1 - sx);
+        b[0] = b0[0] + b0[-sx] + b0[-sxy] + b0[-sx - sxy];
+        b[1] = b1[0] + b1[-1] + b1[-sxy] + b1[-1 - sxy];
+        b[2] = b2[0] + b2[-1] + b2[-sx] + b2[-1 - sx];
     }
 }
 
