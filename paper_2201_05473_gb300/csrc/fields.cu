@@ -23,9 +23,18 @@ namespace {
 constexpr int kBX = PWFA_FIELD_BX;
 constexpr int kBY = PWFA_FIELD_BY;
 
+// The separate Faraday launch (periodic grids below 4 Mi nodes, the PIC driver,
+// FUSION_OFF, the step before a window move). It waits for its predecessor but
+// does not announce the fluid kernel behind it: with the announcement every
+// step of separate field kernels was slower, with Ampere's (whose successor
+// needs a third of the fluid's registers) none. Whole steps on GB300, us,
+// announced / not / all launches plain: 512x256x256 BGK FP32 3746 / 3683 /
+// 3685, regularized FP16 2363 / 2300 / 2308; 256x128x128 476 / 468 / 476;
+// 203x97x131 periodic 320 / 308 / 316; 64x32x32 10.3 / 9.9 / 16.4, FP16
+// 11.6 / 9.4 / 16.4.
 template <bool PER>
 __global__ void __launch_bounds__(kBX * kBY) faraday_kernel(const StepArgs a) {
-    chain_begin();
+    chain_wait();
     const int i = blockIdx.x * kBX + threadIdx.x;
     const int j = blockIdx.y * kBY + threadIdx.y;
     if (i >= a.g.nx || j >= a.g.ny) return;

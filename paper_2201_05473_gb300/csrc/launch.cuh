@@ -3,9 +3,11 @@
 //
 // A chained kernel calls chain_begin() before it touches global memory. The
 // hardware may bring its blocks up once every block of the kernel before has
-// started, and holds them in chain_begin until that kernel has completed and
-// its writes are visible: the same order as a plain launch, without the
-// launch latency and the ramp between the two. Behind a kernel that is not
+// started (and called chain_begin), and holds them there until that kernel has
+// completed and its writes are visible: the same order as a plain launch,
+// without the launch latency and the ramp between the two. With chain_wait()
+// alone a kernel does not let its successor in before it completes, which is
+// the faster form ahead of the fluid kernel (faraday_kernel). Behind a kernel that is not
 // chained, a copy or an event the launch is ordered as usual.
 //
 // What makes that order sound: griddepcontrol.wait holds a thread until the
@@ -24,9 +26,11 @@
 
 namespace pwfa {
 
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ void chain_begin() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    chain_wait();
 }
 
 template <class... P, class... A>
