@@ -57,7 +57,9 @@ constexpr int kPairs = 1024;
 int validate(const pwfa_axi_params& p) {
     auto bad = [](const char* what) { return set_error(PWFA_ERR_PARAM, std::string("axisymmetric: ") + what); };
     if (p.nz < 3 || p.nr < 3) return bad("nz, nr must be >= 3");
-    if ((int64_t)p.nz * p.nr * 27 >= ((int64_t)1 << 40)) return bad("grid too large");
+    // the kernels find (k, j) from 32-bit node indices (FastDiv: below 2^31);
+    // 2^31 nodes of 276 B would be 593 GB
+    if ((int64_t)p.nz * p.nr >= ((int64_t)1 << 31)) return bad("grid too large (nodes >= 2^31)");
     if (!(p.dx > 0) || !std::isfinite(p.dx)) return bad("dx must be > 0");
     if (!(p.dt >= 0) || !std::isfinite(p.dt)) return bad("dt must be >= 0 (0 = default)");
     const double dt = p.dt > 0 ? p.dt : 0.17628 * p.dx;

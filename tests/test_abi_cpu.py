@@ -135,3 +135,14 @@ def test_noalloc_argument_checks(lib):
     assert call(dx=0.0) == -1
     assert call(n_floor=-1.0) == -1 and "n_floor" in lib.pwfa_lbm_last_error().decode()
     assert call(n_floor=float("nan")) == -1
+
+
+@pytest.mark.parametrize("nz,nr", [(1 << 16, 1 << 15), (3, 1 << 30), (200000, 150000)])
+def test_axi_grid_past_32bit_indices_rejected(lib, nz, nr):
+    """The axisymmetric kernels index nodes below 2^31; larger grids are
+    refused before any CUDA call."""
+    p = lbm.AxiParams(nz=nz, nr=nr, dx=0.1, dt=0.0, tau=0.6, collision=0, couple=1, n0=1.0, alpha=0.1,
+                      sigma_r=0.5, sigma_z=0.5, z0=1.0, n_floor=0.0)
+    h = ctypes.c_void_p()
+    assert lib.pwfa_axi_create(ctypes.byref(p), None, ctypes.byref(h)) == -1 and not h.value
+    assert "grid too large" in lib.pwfa_lbm_last_error().decode()
