@@ -942,6 +942,17 @@ int record_instance(pwfa_lbm* h, Instance& in, int32_t nsteps, int32_t ckpt_ever
     cudaStream_t s = h->stream;
     if (in.p.moving_window) return fail(PWFA_ERR_PARAM, "the adjoint does not support the moving window");
     if (in.p.driver != PWFA_DRIVER_RIGID) return fail(PWFA_ERR_PARAM, "the adjoint needs the rigid driver");
+    // While the caller captures the stream nothing runs, so the handle would
+    // hold a recording that never happened. A recording that allocates is
+    // refused by the runtime; one that takes over the allocations of the one
+    // before asks it for a byte first, so that the same captures refuse it.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    PWFA_CUDA(cudaStreamIsCapturing(s, &capture), "cudaStreamIsCapturing");
+    if (capture != cudaStreamCaptureStatusNone) {
+        void* probe = nullptr;
+        if (dev_alloc(&probe, 1) != cudaSuccess) return alloc_fail("recording under stream capture");
+        cudaFree(probe);
+    }
     auto& r = in.rec;
     r.valid = false;
     r.filled = -1;
