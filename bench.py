@@ -370,6 +370,7 @@ def run_ours(args):
             torch.cuda.empty_cache()
             wf = W.production()
             sim = lbm.Simulation(wf, stream=stream)
+            sim.set_launch(*launch_shape)
             barrier()
             with ClockSampler(dev) as fclk:
                 ev0.record(stream)
@@ -486,6 +487,7 @@ def run_ours(args):
             xp, pwt = W.bunch_particles(npart, wp.alpha, wp.sigma_r, wp.sigma_z, wp.z0, wp.dt, wp.nx, wp.ny, wp.dx)
             sp = lbm.Simulation(wp, stream=stream)
             sp.set_particles(xp, pwt)
+            sp.set_launch(*launch_shape)
             sp.step(args.warmup)
             barrier()
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -675,7 +677,10 @@ def run_ours(args):
                    "prelude_steps": args.prelude,
                    "l2": "inputs larger than L2 (populations %.1f GB)" % (2 * 76 * (4 if w.storage == W.F32 else 2) * N / 1e9),
                    "parallelism": "replicas" if world > 1 else "single GPU",
-                   "fluid_block": list(launch_shape), "fluid_variant": fluid_variant},
+                   "fluid_block": list(launch_shape), "fluid_variant": fluid_variant,
+                   "fluid_nodes": ("runs of 128 consecutive nodes"
+                                   if tuple(launch_shape) == (64, 2) and fluid_variant == "direct"
+                                   else "blocks of a plane")},
         "pct_hbm_step": {"of_" + peak_kind: value / world * 1e9 * step_bytes / (peak * 1e9),
                          "of_nominal_8000": value / world * 1e9 * step_bytes / (NOMINAL_HBM_GBS * 1e9),
                          "bytes_per_node_step": step_bytes},

@@ -304,9 +304,12 @@ int pwfa_lbm_profile(pwfa_lbm_t* h, int32_t enable);
 int pwfa_lbm_kernel_times(pwfa_lbm_t* h, double* ms, int64_t* launches);
 
 /* Thread-block shape (bx * by threads, bx along x) of the fused fluid kernel
- * for one instance, in place of the default blocks of 128 consecutive nodes
- * (which fit any row length; get_launch then reports 64 x 2). bx, by >= 1, bx * by a multiple of 32 and at most 128;
- * PWFA_ERR_PARAM otherwise. */
+ * for one instance. 64 x 2, the default, stands for blocks of 128 consecutive
+ * nodes, which fit any row length; other shapes are bx x by nodes of a plane.
+ * What get_launch reports gives another handle the same blocks.
+ * pwfa_lbm_step_diag's last step, pwfa_lbm_record's last segment and the
+ * batched path always take consecutive nodes. bx, by >= 1, bx * by a multiple
+ * of 32 and at most 128; PWFA_ERR_PARAM otherwise. */
 int pwfa_lbm_set_launch(pwfa_lbm_t* h, int32_t instance, int32_t bx, int32_t by);
 int pwfa_lbm_get_launch(pwfa_lbm_t* h, int32_t instance, int32_t* bx, int32_t* by);
 

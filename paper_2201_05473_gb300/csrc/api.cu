@@ -79,9 +79,8 @@ struct Instance {
     double* d_wout = nullptr;   // witness slab: FP64 sum of E_z
     unsigned* d_dbg = nullptr;  // debug builds: index-error word (site, index, count)
     int64_t steps = 0;
-    // fluid kernel blocks: runs of 128 nodes, or bx x by nodes of a plane once
-    // pwfa_lbm_set_launch or the autotuner has chosen a shape
-    bool linear = true;
+    // fluid kernel blocks: bx x by nodes of a plane, 64 x 2 standing for runs
+    // of 128 consecutive nodes (takes_runs)
     int bx = 64, by = 2;
     int variant = PWFA_FLUID_DIRECT;  // fluid kernel variant
     // recording for the adjoint: checkpoints every K steps (+ the final
@@ -232,6 +231,12 @@ int check_instance(pwfa_lbm* h, int32_t i) {
     return PWFA_OK;
 }
 
+// The direct fluid kernel's blocks. 64 x 2 names the runs, so that what
+// get_launch reports of a default or autotuned instance gives another one the
+// same kernel through set_launch; as a block shape 64 x 2 was slower at every
+// size measured (LinearMap).
+bool takes_runs(int bx, int by) { return bx == 64 && by == 2; }
+
 StepArgs make_args(const Instance& in) {
     StepArgs a{};
     a.g = in.g;
@@ -263,7 +268,7 @@ StepArgs make_args(const Instance& in) {
     a.dx = (float)p.dx;
     a.bx = in.bx;
     a.by = in.by;
-    a.linear = in.linear;
+    a.linear = takes_runs(in.bx, in.by);
     a.staged = in.variant == PWFA_FLUID_STAGED && in.bx * in.by == 128;
     a.dbg = in.d_dbg;
     for (int c = 0; c < 3; ++c) a.Jb[c] = in.Jb[c];
@@ -1602,7 +1607,6 @@ int pwfa_lbm_set_launch(pwfa_lbm_t* h, int32_t instance, int32_t bx, int32_t by)
     if (rc) return rc;
     if (bx < 1 || by < 1 || bx * by > PWFA_FLUID_MAX_THREADS || (bx * by) % 32)
         return fail(PWFA_ERR_PARAM, "block shape must be a multiple of 32 threads, at most 128");
-    h->inst[instance].linear = false;
     h->inst[instance].bx = bx;
     h->inst[instance].by = by;
     h->batch_valid = false;
@@ -1636,12 +1640,10 @@ int pwfa_lbm_get_launch(pwfa_lbm_t* h, int32_t instance, int32_t* bx, int32_t* b
 int pwfa_lbm_autotune(pwfa_lbm_t* h, int32_t reps) {
     if (!h) return fail(PWFA_ERR_PARAM, "null handle");
     if (reps < 1) return fail(PWFA_ERR_PARAM, "reps must be >= 1");
-    // {bx, by, variant, linear}: runs of consecutive nodes, direct shapes,
-    // then the staged kernel's 128-thread tiles (the batched path's per-node
-    // phases take runs of nodes too; the choice serves the per-instance
-    // steps)
-    static const int cand_all[][4] = {{64, 2, 0, 1}, {32, 4, 0, 0}, {64, 2, 0, 0}, {128, 1, 0, 0},
-                                      {32, 4, 1, 0}, {64, 2, 1, 0}, {128, 1, 1, 0}};
+    // {bx, by, variant}: runs of consecutive nodes, direct shapes, then the
+    // staged kernel's 128-thread tiles (the batched path's per-node phases
+    // take runs of nodes too; the choice serves the per-instance steps)
+    static const int cand_all[][3] = {{64, 2, 0}, {32, 4, 0}, {128, 1, 0}, {32, 4, 1}, {64, 2, 1}, {128, 1, 1}};
     const int ncand = (int)(sizeof cand_all / sizeof cand_all[0]);
     h->batch_valid = false;
     cudaEvent_t e0, e1;
@@ -1650,15 +1652,15 @@ int pwfa_lbm_autotune(pwfa_lbm_t* h, int32_t reps) {
     int rc = PWFA_OK;
     for (auto& in : h->inst) {
         float best = 1e30f;
-        int bb[4] = {in.bx, in.by, in.variant, in.linear};
+        int bb[3] = {in.bx, in.by, in.variant};
         for (int ci = 0; ci < ncand; ++ci) {
             const int* c = cand_all[ci];
-            if (!c[3] && c[0] > 2 * in.g.nx && c[0] > 32) continue;  // mostly idle lanes
+            const bool runs = takes_runs(c[0], c[1]) && c[2] == PWFA_FLUID_DIRECT;
+            if (!runs && c[0] > 2 * in.g.nx && c[0] > 32) continue;  // mostly idle lanes
             if (c[0] * c[1] > PWFA_FLUID_MAX_THREADS) continue;
             in.bx = c[0];
             in.by = c[1];
             in.variant = c[2];
-            in.linear = c[3] != 0;
             StepArgs a = make_args(in);
             a.src_shift = 0;  // time a plain step even if the next one moves the window
             cudaError_t e = launch_fluid(a, in.p.storage, in.p.collision, h->stream);  // warm
@@ -1669,12 +1671,11 @@ int pwfa_lbm_autotune(pwfa_lbm_t* h, int32_t reps) {
             float ms = 0.0f;
             if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
             if (e != cudaSuccess) { rc = cuda_fail(e, "autotune"); break; }
-            if (ms < best) { best = ms; bb[0] = c[0]; bb[1] = c[1]; bb[2] = c[2]; bb[3] = c[3]; }
+            if (ms < best) { best = ms; bb[0] = c[0]; bb[1] = c[1]; bb[2] = c[2]; }
         }
         in.bx = bb[0];
         in.by = bb[1];
         in.variant = bb[2];
-        in.linear = bb[3] != 0;
         if (rc) break;
     }
     cudaEventDestroy(e0);

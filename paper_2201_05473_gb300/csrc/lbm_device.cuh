@@ -253,7 +253,7 @@ struct StepArgs {
                           // that moves the window (the streaming source is
                           // read one plane up), else 0
     int bx, by;           // fluid kernel block shape (autotuned per instance)
-    int linear;           // 1: blocks of 128 consecutive nodes instead of bx x by (LinearMap)
+    int linear;           // 1: blocks of 128 consecutive nodes instead of bx x by (LinearMap); bx x by is 64 x 2
     int staged;           // 1: software-pipelined fluid kernel (FP32 storage), 128-thread tiles
     unsigned* dbg;        // debug builds: the instance's index-error word (see PWFA_CHECK)
     float* mom;           // adjoint recompute (launch_fluid_mom): each node's lattice

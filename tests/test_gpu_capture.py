@@ -4,8 +4,10 @@ its own. pwfa_lbm_step may be captured: its launches, chained to one another
 of the field step. pwfa_lbm_record may not, whether it would allocate or take
 over an earlier recording's allocations: it returns PWFA_ERR_CUDA and the
 earlier recording stays usable."""
+import ctypes
 import json
 import os
+import re
 import subprocess
 import sys
 
@@ -98,3 +100,35 @@ def test_record_is_refused_under_capture(recorded):
     r = json.loads([ln for ln in cp.stdout.splitlines() if ln.startswith("RESULT ")][-1][len("RESULT "):])
     assert r["code"] == -2 and "captur" in r["msg"].lower(), r  # PWFA_ERR_CUDA
     assert r.get("equal"), r
+
+
+def fluid_kernels(sim, stream, path):
+    """Names of the fluid kernels that one step launches, from a capture of
+    the step."""
+    rt = ctypes.CDLL("libcudart.so.%s" % torch.version.cuda.split(".")[0])
+    st, graph = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p()
+    assert rt.cudaStreamBeginCapture(st, 1) == 0
+    sim.step(1)
+    assert rt.cudaStreamEndCapture(st, ctypes.byref(graph)) == 0
+    assert rt.cudaGraphDebugDotPrint(graph, str(path).encode(), 1) == 0
+    assert rt.cudaGraphDestroy(graph) == 0
+    return set(re.findall(r"fluid_(?:linear_|staged_)?kernel", path.read_text()))
+
+
+def test_launch_shape_round_trip(tmp_path):
+    """What get_launch reports gives another handle the same kernel: the
+    default's runs of nodes, and a block shape."""
+    w = W.parity_small().replace(nx=131, ny=24, nz=24, storage=W.F16, collision=W.REGULARIZED)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st), lbm.Simulation(w, stream=st) as a, lbm.Simulation(w, stream=st) as b:
+        for shape, kernel in ((None, "fluid_linear_kernel"), ((32, 4), "fluid_kernel"),
+                              ((64, 2), "fluid_linear_kernel")):
+            if shape:
+                a.set_launch(*shape)
+            b.set_launch(*a.get_launch())
+            assert b.get_launch() == a.get_launch()
+            a.step(2)
+            b.step(2)
+            st.synchronize()
+            for s in (a, b):
+                assert fluid_kernels(s, st, tmp_path / "step.dot") == {kernel}
