@@ -504,10 +504,13 @@ static cudaError_t diag_t(const StepArgs& a, int blocks, double dxcube, double* 
 
 cudaError_t launch_diag(const StepArgs& a, int storage, double dxcube, double* partials, double* out, cudaStream_t s) {
     const int64_t need = (a.g.N + kDiagThreads - 1) / kDiagThreads;
-    constexpr int64_t resident = 2 * 152;  // two blocks per SM
-    static_assert(resident <= kDiagBlocks, "partial records");
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
+    // two blocks per SM, a partial record each
+    const int64_t resident = 2 * sms < kDiagBlocks ? 2 * sms : kDiagBlocks;
     const int blocks = (int)(need < resident ? need : resident);
-    cudaError_t e = cudaErrorInvalidValue;
+    e = cudaErrorInvalidValue;
     switch (storage) {
         case 0: e = diag_t<0>(a, blocks, dxcube, partials, s); break;
         case 1: e = diag_t<1>(a, blocks, dxcube, partials, s); break;

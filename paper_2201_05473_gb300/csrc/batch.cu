@@ -75,9 +75,8 @@ __global__ void __launch_bounds__(kBatchTile, PHASE == 1 ? BatchFluidOcc<ST, COL
     }
 }
 
-// Phase 3 on the fused-field tiles: Ampere of this step with Faraday of the
-// next.
-template <bool PER>
+// Phase 3 on the fused-field tiles (periodic grids): Ampere of this step with
+// Faraday of the next.
 __global__ void __launch_bounds__(kAFX * kAFY, PWFA_AF_MIN_BLOCKS)
     batch_fields_kernel(const BatchEntry* __restrict__ ent, const uint16_t* __restrict__ ftile_inst, int parity) {
     __shared__ StepArgs sa;
@@ -95,7 +94,7 @@ __global__ void __launch_bounds__(kAFX * kAFY, PWFA_AF_MIN_BLOCKS)
     const int tbz = (int)(local / per_slab);
     const int r = (int)(local - (int64_t)tbz * per_slab);
     const int tby = r / e.ftiles_x;
-    ampere_faraday_tile<PER>(sa, so, r - tby * e.ftiles_x, tby, tbz, s_zc);
+    ampere_faraday_tile<true>(sa, so, r - tby * e.ftiles_x, tby, tbz, s_zc);
 }
 
 // The same on open grids, on rows of nodes: a block takes four consecutive
@@ -146,8 +145,8 @@ cudaError_t launch_phase(const BatchLaunch& b, int phase, int parity, cudaStream
         case 2: batch_node_kernel<ST, COLL, PER, 2><<<nt, kBatchTile, 0, s>>>(b.entries, b.tile_inst, parity); break;
         case 3:
             if (PER)
-                batch_fields_kernel<PER><<<(unsigned)b.nftiles, dim3(kAFX, kAFY, 1), 0, s>>>(b.entries, b.ftile_inst,
-                                                                                             parity);
+                batch_fields_kernel<<<(unsigned)b.nftiles, dim3(kAFX, kAFY, 1), 0, s>>>(b.entries, b.ftile_inst,
+                                                                                        parity);
             else
                 batch_rows_kernel<<<(unsigned)b.nftiles, kARThreads, 0, s>>>(b.entries, b.ftile_inst, parity);
             break;

@@ -127,7 +127,7 @@ cudaError_t launch_rows_h(const StepArgs& a, const FieldPair& out, cudaStream_t 
 // consecutive nodes per thread were slower (63 us at 256x128x128: 157
 // registers), and so were blocks of 256 or 384 threads and seven or eight
 // blocks per SM (spills). Planes: the fewest whose blocks the GPU holds at
-// once, up to four (128x64x64: 14.6, 13.1, 14.2 us with 2, 3, 4; 256x128x128
+// once, two (one never fits from 256 Ki nodes on) to four (128x64x64: 14.6, 13.1, 14.2 us with 2, 3, 4; 256x128x128
 // 87, 61.5, 59, 57 with 1 to 4, 61 with 8); eight from 8 Mi nodes on
 // (512x256x256: 377 with 4, 371).
 //
@@ -140,11 +140,13 @@ cudaError_t launch_rows(const StepArgs& a, const FieldPair& out, cudaStream_t s)
         if (a.g.N < ((int64_t)96 << 10)) return launch_rows_h<1, 1>(a, out, s);
         return a.g.N < ((int64_t)640 << 10) ? launch_rows_h<1, 2>(a, out, s) : launch_rows_h<1, 4>(a, out, s);
     }
-    auto fits = [&](int h) {
-        return rows_blocks(a.g, 2) * (int64_t)((a.g.nz + h - 1) / h) <= 152 * kARBlocks<2>;
-    };
     if (a.g.N >= kTileNodes) return launch_rows_h<2, 8>(a, out, s);
-    if (fits(1)) return launch_rows_h<2, 1>(a, out, s);
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
+    auto fits = [&](int h) {
+        return rows_blocks(a.g, 2) * (int64_t)((a.g.nz + h - 1) / h) <= (int64_t)sms * kARBlocks<2>;
+    };
     if (fits(2)) return launch_rows_h<2, 2>(a, out, s);
     if (fits(3)) return launch_rows_h<2, 3>(a, out, s);
     return launch_rows_h<2, 4>(a, out, s);

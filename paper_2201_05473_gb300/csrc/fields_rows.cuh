@@ -2,7 +2,7 @@
 // n + 1) over runs of consecutive nodes. Bodies of the separate updates:
 // fields_node.cuh; the same step over tiles: fields_fused.cuh.
 //
-// A warp takes 31 V consecutive nodes of a plane, V (1, 2 or 4; a divisor of
+// A warp takes 31 V consecutive nodes of a plane, V (1 or 2; a divisor of
 // nx) per thread, and marches up H planes. Each thread evaluates E_{n+3/2} at
 // its nodes, plane by plane; of the three neighbours' E that Faraday reads,
 // the +x one comes from the thread itself or the next lane (lane 31 only
@@ -27,10 +27,7 @@ constexpr int kARLanes = 31;
 // V consecutive nodes' values as one load or store (p aligned to V floats)
 template <int V>
 __device__ __forceinline__ void row_ld(float (&d)[V], const float* p) {
-    if constexpr (V == 4) {
-        const float4 t = ld_state(reinterpret_cast<const float4*>(p));
-        d[0] = t.x; d[1] = t.y; d[2] = t.z; d[3] = t.w;
-    } else if constexpr (V == 2) {
+    if constexpr (V == 2) {
         const float2 t = ld_state(reinterpret_cast<const float2*>(p));
         d[0] = t.x; d[1] = t.y;
     } else {
@@ -39,8 +36,7 @@ __device__ __forceinline__ void row_ld(float (&d)[V], const float* p) {
 }
 template <int V>
 __device__ __forceinline__ void row_st(float* p, const float (&d)[V]) {
-    if constexpr (V == 4) *reinterpret_cast<float4*>(p) = make_float4(d[0], d[1], d[2], d[3]);
-    else if constexpr (V == 2) *reinterpret_cast<float2*>(p) = make_float2(d[0], d[1]);
+    if constexpr (V == 2) *reinterpret_cast<float2*>(p) = make_float2(d[0], d[1]);
     else *p = d[0];
 }
 // The +x / -x neighbours' values of V consecutive ones. With V = 1 what was

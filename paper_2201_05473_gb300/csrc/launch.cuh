@@ -33,6 +33,13 @@ __device__ __forceinline__ void chain_begin() {
     chain_wait();
 }
 
+// Multiprocessors of the current device.
+inline cudaError_t sm_count(int* n) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e == cudaSuccess ? cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev) : e;
+}
+
 template <class... P, class... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A&&... args) {
     cudaLaunchAttribute attr{};
