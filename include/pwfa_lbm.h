@@ -150,13 +150,17 @@ int pwfa_lbm_step(pwfa_lbm_t* h, int32_t nsteps);
  * pwfa_lbm_record resets the instance to its initial condition (t = 0) and
  * advances it nsteps, keeping a checkpoint of the full state every
  * ckpt_every steps (0 selects ceil(sqrt(nsteps)), or nsteps, one segment,
- * where that takes no more memory: up to some 65 steps in FP32, 20 in 16-bit
- * storage) plus the final state. The instance is left at step nsteps. Device memory: (nsteps/ckpt_every + 1)
- * states of 76 N populations + 6 N field values; one segment of K =
- * ckpt_every recomputed steps (two population buffers, the E and B of its
- * states, 6 (K + 1) N values, and the four lattice sums of each step, 4 K N:
- * the reverse step needs nothing else of the populations); ~174 N floats of
- * adjoint scratch; PWFA_ERR_ALLOC if it does not fit. The last segment
+ * where that takes no more memory: the two sizes are compared, and one segment
+ * is the smaller up to about 65 steps in FP32 and 18 in 16-bit storage) plus
+ * the final state. The instance is left at step nsteps. Device memory, kept
+ * for the next recording of the instance unless that needs less than half of
+ * it or more than there is: (nsteps/ckpt_every + 1) states of 76 N populations
+ * + 6 N field values; one segment of K = ckpt_every recomputed steps (two
+ * population buffers, the E and B of its states, 6 (K + 1) N values, and the
+ * four lattice sums of each step, 4 K N: the reverse step needs nothing else
+ * of the populations); ~174 N floats of adjoint scratch; PWFA_ERR_ALLOC if it
+ * does not fit, PWFA_ERR_CUDA while the caller captures the stream in a mode
+ * that forbids allocations. The last segment
  * runs as the reverse sweep would recompute it, into the segment storage,
  * so the next pwfa_lbm_adjoint_step reverses it without recomputing it; with
  * ckpt_every >= nsteps (one segment of nsteps steps, when memory allows)

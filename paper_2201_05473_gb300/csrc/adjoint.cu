@@ -5,12 +5,14 @@
 //   Bn     = Bc - c curl E                              (Faraday, active faces)
 //   S^n, J = fluid(S^{n-1}, E, Bc, Bn)                  (stream+collide+source)
 //   E'     = E + c curl Bn - dt (avg J + J_b(theta))    (Ampere, active edges)
-// Reverse step n, given the adjoints of (S^n, E', Bn as the next B):
+// Reverse step n, given the adjoints of (f^{n+1}, the pre-collision populations
+// that step n + 1 pulled from S^n; E'; Bn as the next B):
 //   R1  adj_ampere:   Bn_bar += c curl^T(E'_bar); J_bar = -dt avg^T(E'_bar);
 //                     theta_bar += dt E'_z,bar dJ_b/dtheta (FP64)
 //   R2a adj_fluid (boundary nodes): A_bar of each Eq. 14 boundary node
-//   R2  adj_fluid (interior nodes): S^{n-1}_bar by the transposed pull
-//                     (a scatter to x - xi_i), node E_bar and B_bar
+//   R2  adj_fluid (interior nodes): gathers S^n_bar,i(x) = f^{n+1}_bar,i(x + xi_i)
+//                     (the transposed pull), gives f^n_bar at its own node,
+//                     node E_bar and B_bar
 //   R3  adj_faces:    Bn_bar += avg4^T(b_bar)/8; Bc_bar = Bn_bar + avg4^T(b_bar)/8
 //   R4  adj_edges:    E_bar = E'_bar + avg2^T(e_bar)/2 - c curl_F^T(Bn_bar)
 // with c = dt/dx. All adjoint state is FP32; parameter gradients are FP64.
@@ -437,7 +439,12 @@ __global__ void __launch_bounds__(kLinearThreads, 4) adj_fluid_kernel(const AdjA
     // sum w S (xi.u)^2 = u.W), and its share of u_bar, through
     // phi_i = w_i (base + 3 xi.u + 4.5 (xi.u)^2) and the regularized
     // projection's -k3 A_l P_l. Every lattice's share is rounded before it is
-    // added (no fused multiply-add), whichever thread forms it.
+    // added. The roundings marked here and below (this one, the mean of E, the
+    // sums of the moment adjoints) are not the method's: they are those of the
+    // form that gave each lattice a warp and passed the shares through memory,
+    // kept so that gradients, FP64 numbers from FP32 adjoints, stay the same
+    // from version to version. Another form of the sums above moved them by
+    // 2.4e-9 of themselves and would have saved 8 of 517 us.
     float Ab[kL], Gs[3], ub[3];
     float mk[kL][3];  // (regularized: for the populations' adjoints)
 #pragma unroll
@@ -474,7 +481,7 @@ __global__ void __launch_bounds__(kLinearThreads, 4) adj_fluid_kernel(const AdjA
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 b[c] = 0.125f * (bc[c] + bn[c]);
-                asm("" : "+f"(e[c]));  // the mean is rounded before it is used
+                asm("" : "+f"(e[c]));  // (rounded before it is used: see above)
             }
             F[0] = -n * (e[0] + beta[1] * b[2] - beta[2] * b[1]);
             F[1] = -n * (e[1] + beta[2] * b[0] - beta[0] * b[2]);
@@ -535,8 +542,8 @@ __global__ void __launch_bounds__(kLinearThreads, 4) adj_fluid_kernel(const AdjA
         }
         if (n > s.n_floor) nb += nnb;
         // ---- the moment adjoints
-        // (on periodic BGK grids, where omega weights every node, the weight
-        // and the sum are one fused multiply-add)
+        // (rounded as said above; on periodic BGK grids, where omega weights
+        // every node, weight and sum had been one fused multiply-add)
         auto plus = [&](float v, float own) { return PER && COLL == 0 ? __fmaf_rn(wA, own, v) : __fadd_rn(v, own); };
         Ab[0] = plus(nb, Ab[0]);
 #pragma unroll

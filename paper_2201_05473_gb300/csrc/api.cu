@@ -728,9 +728,10 @@ int step_instance(pwfa_lbm* h, Instance& in, const DiagOut* diag) {
 
 // ---------------------------------------------------------------- adjoint
 // One segment of a recording: the two population buffers the recomputed
-// forward steps ping-pong between (the first step reads its checkpoint), then E of each of its K states and B of
-// its K + 1 states (each field array behind a zero guard), and the lattice
-// sums A_l ([4][N]) that each recomputed step stores for the reverse step.
+// forward steps ping-pong between (the first step reads its checkpoint), then
+// E of each of its K states and B of its K + 1 states (each field array behind
+// a zero guard), and the lattice sums A_l ([4][N]) that each recomputed step
+// stores for the reverse step.
 struct SegLayout {
     size_t fb, vb, gvb, gb;
     int64_t K;
@@ -931,9 +932,11 @@ int fill_segment(pwfa_lbm* h, Instance& in, int seg) {
 // or nsteps (one segment, nothing recomputed) where that takes no more
 // memory. A step kept in a segment is its fields and lattice sums, 40 B a
 // node; a checkpoint also holds the populations, 328 B (FP32) or 176, and
-// saves what lies between. So one segment is the smaller up to 65 (FP32) or 22
-// (16-bit) steps: 40 steps of 256x128x128 take 12.0 instead of 13.4 GB, and
-// record + sweep 45 instead of 62.6 ms.
+// saves what lies between. The sizes are compared as they come out, which is
+// no single line because ceil(sqrt) jumps: 256x128x128 runs as one segment up to
+// 66 steps and at 73 and 74 (FP32), up to 18 and at 21 and 22 (16-bit). 40 FP32
+// steps of it take 12.1 instead of 13.4 GB, and record + sweep 45 instead of
+// 62.6 ms.
 int default_interval(const Instance& in, int32_t nsteps) {
     const int32_t K = std::min((int32_t)std::ceil(std::sqrt((double)nsteps)), nsteps);
     auto bytes = [&](int32_t k) {
@@ -973,7 +976,7 @@ int record_instance(pwfa_lbm* h, Instance& in, int32_t nsteps, int32_t ckpt_ever
                              align_up(sizeof(double) * (260 + 3 * kGradSlots));
     // The recording before leaves its allocations to this one unless they are
     // too small, or more than twice too large (releasing and allocating the
-    // 18 GB of a 40-step recording of 256x128x128 took 12 of 35 ms).
+    // 16.3 GB of 40 steps of 256x128x128 with checkpoints took 12 of 35 ms).
     auto fits = [](const void* p, size_t have, size_t need) { return p && have >= need && have / 2 <= need; };
     if (!fits(r.cp, r.cp_bytes, cp_bytes) || !fits(r.seg, r.seg_bytes, seg_bytes) ||
         !fits(r.adj, r.adj_bytes, adj_bytes)) {

@@ -154,7 +154,7 @@ template <> struct Codec<2> {
 // replaced by lo, so nothing outside the allocation is read or written; the
 // host then fails the call with PWFA_ERR_STATE. Release builds compile the
 // checks away. Sites: 1 pulled source node, 2 stored node, 3 node-average
-// field read, 4 Faraday, 5 Ampere, 6 fused field step, 7 adjoint scatter.
+// field read, 4 Faraday, 5 Ampere, 6 fused field step, 7 adjoint gather.
 #ifdef PWFA_DEBUG
 static __device__ __noinline__ void debug_record(unsigned* dbg, unsigned site, long long i) {
     if (!dbg) return;
