@@ -30,7 +30,7 @@ constexpr int kBY = PWFA_FIELD_BY;
 // needs a third of the fluid's registers) none. Whole steps on GB300, us,
 // announced / not / all launches plain: 512x256x256 BGK FP32 3746 / 3683 /
 // 3685, regularized FP16 2363 / 2300 / 2308; 256x128x128 476 / 468 / 476;
-// 203x97x131 periodic 320 / 308 / 316; 64x32x32 10.3 / 9.9 / 16.4, FP16
+// 131x97x203 periodic 320 / 308 / 316; 64x32x32 10.3 / 9.9 / 16.4, FP16
 // 11.6 / 9.4 / 16.4.
 template <bool PER>
 __global__ void __launch_bounds__(kBX * kBY) faraday_kernel(const StepArgs a) {

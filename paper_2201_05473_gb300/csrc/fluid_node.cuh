@@ -96,7 +96,7 @@ constexpr int kStashVals = 2 * kQ;
 // regularized 3176 / 3138 us, 256x128x128 BGK 408 / 406, 203x97x131 254.8 /
 // 253.6; 32 batched instances 5358 / 5417. So with separate field kernels:
 // whole steps, 512x256x256 with 2e5 particles 3797 / 3782, FUSION_OFF 3722 /
-// 3705, periodic 203x97x131 322.9 / 320.2.
+// 3705, periodic 131x97x203 322.9 / 320.2.
 template <bool CS>
 __device__ __forceinline__ void put(float* p, float v) {
     if (CS) __stcs(p, v);

@@ -20,7 +20,7 @@ constexpr int kPop = kQ * kL;
 // ones. A chained kernel's blocks may be resident while its predecessor still
 // writes what they are going to read (launch.cuh); the read-only path of
 // __ldg is documented for data that nothing writes while the kernel runs.
-// Opaque, so that they stay in program order behind the wait. 203x97x131 BGK
+// Opaque, so that they stay in program order behind the wait. 131x97x203 BGK
 // 289.2 us per step with __ldg, 289.7 with these; 512x256x256 regularized,
 // 256x128x128 BF16 and the field kernels the same to 0.1 %.
 __device__ __forceinline__ float ld_state(const float* p) {

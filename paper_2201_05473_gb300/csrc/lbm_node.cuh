@@ -152,7 +152,7 @@ __device__ __forceinline__ float yat(const Grid& g, const float* a, int i, int j
 // zero, so the indices just below the grid (x-1, y-1, z-1 and their
 // combinations, wrapping into the previous row/plane or the guard) read 0.
 // Plain loads, coherent as ld_state's but the compiler's to place: opaque ones
-// here cost the BGK form 2 to 4 % (203x97x131 FP32 289.2 -> 297.2 us per step,
+// here cost the BGK form 2 to 4 % (131x97x203 FP32 289.2 -> 297.2 us per step,
 // 256x128x128 BF16 310 -> 323).
 template <bool PER>
 __device__ __forceinline__ void node_E(const Grid& g, const float* const E[3], int x, int y, int z, float e[3],
